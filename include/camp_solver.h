@@ -122,8 +122,8 @@ camp_status camp_solver_set_stream(camp_solver_t h, void *stream);
  *                   per CTA (the last CTA takes the remainder).
  *   CAMP_ARR_AUTO : library choice.
  * With 16 lanes per cell (the automatic choice for 33 to 80 species), a
- * launch whose pairs would keep at most a quarter of the GPU's resident warps
- * busy solves each cell alone on a warp instead, on a split of the 16-lane
+ * launch whose pairs would keep at most three quarters of the GPU's resident
+ * warps busy (a third in camp_solver_solve_host's chunks) solves each cell alone on a warp instead, on a split of the 16-lane
  * layout that performs the same operations in the same order: the results
  * are bit for bit those of the pair solve, and a small batch finishes about
  * a fifth sooner.
@@ -356,8 +356,8 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
  * slot: word0 = the entry k (pattern order) whose value the slot multiplies,
  * or 0xFFFFFFFF for a padding slot; word1 = column (bits 0-10) | row
  * (bits 11-21) | 1 << 31 on the last entry of a row (store the running sum to
- * that row).  Padding slots contribute zero.  The kernels stage each cell's
- * matrix values in this slot order.  capacity_slots is the number of slots
+ * that row).  Padding slots contribute zero.  The kernels keep every row's
+ * entries in this order; which lane and slots a row gets may differ.  capacity_slots is the number of slots
  * words can hold.  Pattern requirements as for camp_solver_create.
  */
 camp_status camp_schedule_build(int n, int nnz, const int *row_ptr,

@@ -56,6 +56,21 @@ camp_status camp_schedule_build_split(int n, int nnz, const int *row_ptr,
                                       const int *col_idx, unsigned *words,
                                       int capacity_slots, int *slots_per_lane);
 
+/*
+ * The aligned layout the FP64 kernels run a schedule's rows in (host only, no
+ * GPU): the rows of camp_schedule_build at lanes_per_cell lanes, each with its
+ * entries in the same order, packed again so that all lanes end their rows in
+ * a few common slots; split != 0 (lanes_per_cell 16 only): the same rows on
+ * 32 lanes, for a cell alone on a warp.  Layout and arguments as
+ * camp_schedule_build; a padding slot (entry 0xFFFFFFFF) either leads a row
+ * and reads one of the row's own columns, or follows its lane's last row.
+ * *slots_per_lane = 0: no such layout in as few slots (the kernels then keep
+ * the schedule's own).
+ */
+camp_status camp_schedule_build_aligned(int n, int nnz, const int *row_ptr, const int *col_idx,
+                                        int lanes_per_cell, int split, unsigned *words,
+                                        int capacity_slots, int *slots_per_lane);
+
 #ifdef __cplusplus
 }
 #endif

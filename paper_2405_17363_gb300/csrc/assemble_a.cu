@@ -3,8 +3,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 1)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 2)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 3)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 4)
+CAMP_KERNEL_DEFINE(assemble, 1)
+CAMP_KERNEL_DEFINE(assemble, 2)
+CAMP_KERNEL_DEFINE(assemble, 3)
+CAMP_KERNEL_DEFINE(assemble, 4)
 }  // namespace camp

@@ -3,8 +3,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 5)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 6)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 7)
-CAMP_KERNEL_DEFINE(assemble, assemble_bicgstab_kernel, 8)
+CAMP_KERNEL_DEFINE(assemble, 5)
+CAMP_KERNEL_DEFINE(assemble, 6)
+CAMP_KERNEL_DEFINE(assemble, 7)
+CAMP_KERNEL_DEFINE(assemble, 8)
 }  // namespace camp

@@ -7,15 +7,30 @@
 
 namespace camp {
 
-// SpMV schedule slot (see build_schedule in solver.cu), laid out
-// [slot j][lane-in-cell sl] so a cell's lanes read consecutive words:
-//   col (bits 0-10) | row (bits 11-21) | end (bit 31): the slot multiplies the
-//   gathered vector's entry col; on the last slot of a row (end) the running
-//   sum is stored to row.  Alongside, src[j][sl] is the entry of the cell's
-//   A row (pattern order) that slot uses, or -1 for padding: each cell's A is
-//   staged in slot order, so lanes read consecutive shared-memory words.
+// SpMV schedule word of one slot (see build_schedule in solver.cu): 4 * col
+// (bits 16-31) | 4 * row (bits 2-11) | end (bit 0): the slot multiplies the
+// gathered vector's entry col; on the last slot of a row (end) the running
+// sum is stored to row.  Four slots of a lane are one 16-byte load: slot j of
+// lane sl lies at word_pos(j, sl).  Alongside, src (same places) is the entry
+// of the cell's A row (pattern order) that slot uses, or -1 for padding; each
+// cell's A is staged in slot order, two slots of a lane side by side
+// (pair_pos), so a lane reads them with one 16-byte load.  Slots past the last
+// whole block (pair) lie [slot][lane], so neither layout needs padding.
 typedef unsigned int SchedWord;
-constexpr unsigned kSlotEnd = 0x80000000u;
+constexpr unsigned kSlotEnd = 1u, kSlotRowMask = 0xfffcu;
+constexpr int kSlotBlock = 4;  // slots per word block
+// Words of a launch's row-end mask, one bit per slot; slots past it are taken
+// as row ends of some lane (what every slot of so long a product is anyway).
+constexpr int kEndWords = 8;
+__host__ __device__ inline SchedWord slot_word(int col, int row, bool end) {
+  return ((SchedWord)col << 18) | ((SchedWord)row << 2) | (end ? kSlotEnd : 0u);
+}
+__host__ __device__ inline int word_pos(int j, int sl, int L, int Lc) {
+  return j < (L & ~3) ? ((j >> 2) * Lc + sl) * 4 + (j & 3) : j * Lc + sl;
+}
+__host__ __device__ inline int pair_pos(int j, int sl, int L, int Lc) {
+  return j < (L & ~1) ? ((j >> 1) * Lc + sl) * 2 + (j & 1) : j * Lc + sl;
+}
 // Bytes the plain launches reserve at the start of dynamic shared memory for
 // nsch schedule words (rounded to 16); the host sizes the allocation and the
 // kernels place their per-warp regions with this one function.
@@ -38,11 +53,14 @@ struct WarpArgs {
   int *iters;              // [cells]
   double *resid;           // [cells]
   int *status;             // [cells] or null
-  const SchedWord *sched;  // [L x Lc] slot words
-  const int *src;          // [L x Lc] A entry of each slot (transposed view: permuted), -1 pad
-  const int *dst;          // [nnz] slot of each A entry (pattern order): inverse of src
-  const int *padfrom;      // [Lc] first padding slot of each lane
-  const int *dslot;        // [n] slot of each row's diagonal entry
+  const SchedWord *sched;  // [L x Lc] slot words (word_pos)
+  const int *src;          // [L x Lc] A entry of each slot (word_pos; transposed view: permuted), -1 pad
+  const int *dst;          // [nnz] place (pair_pos) of each A entry (pattern order)
+  const int *pads;         // [npads] places (pair_pos) of the padding slots; npads < 0: [Lc] each
+  int npads;               // lane's first padding slot (all its later ones are padding too)
+  unsigned ends[kEndWords];  // bit j: some lane ends a row in slot j
+  const int *dslot;        // [n] place (pair_pos) of each row's diagonal entry
+  const int *dentry;       // [n] A entry of each row's diagonal (A read from global memory)
   // Single-cell tickets (the plain launch at 16 lanes per cell): tickets t <
   // single_from solve the pair at positions 2t, 2t+1; tickets t >= single_from
   // solve the one cell at position 2 * single_from + (t - single_from) with
@@ -53,9 +71,11 @@ struct WarpArgs {
   int single_from;
   int L2;                  // slots per lane of the split schedule
   const SchedWord *sched2; // [L2 x 32]
-  const int *dst2;         // [nnz] split slot of each A entry
-  const int *padfrom2;     // [32] first padding slot of each lane
-  const int *dslot2;       // [n] split slot of each row's diagonal entry
+  const int *dst2;         // [nnz] split place of each A entry
+  const int *pads2;        // [npads2] places of its padding slots
+  int npads2;
+  unsigned ends2[kEndWords];
+  const int *dslot2;       // [n] split place of each row's diagonal entry
   double tol;
   int maxit;
   int x0_given;
@@ -99,13 +119,13 @@ struct WarpArgs {
   long long ord_wait;
   // Fused assembly (assemble_bicgstab_kernel only): the cell's matrix is
   // built in shared memory as A = I - gamma J(conc) instead of read from A.
-  // Lane sl runs tcount terms p: J[slot (tmeta >> 11) * Lc + sl] +=
+  // Lane sl runs tcount terms p: J[place tmeta >> 11] +=
   // tval * (conc[(tmeta & 0x7ff) - 1] or 1 when that field is 0); arrays
   // are laid out [p][lane], padding terms add zero.
   const double *conc;      // [cells x n]
   const double *gamma;     // [cells]
   const double *tval;      // [tcount x Lc] sign * rate constant
-  const int *tmeta;        // [tcount x Lc] species + 1 | slot row << 11
+  const int *tmeta;        // [tcount x Lc] species + 1 | place (pair_pos) << 11
   int tcount;
   // Newton corrector (newton_bicgstab_kernel only): lane sl accumulates
   // f[row sl + e*Lc] += rval * y[a] * (y[b] or 1) over its rcount terms,
@@ -166,8 +186,9 @@ struct GradArgs {
 // co-resident: at most SMs x the occupancy of the launch shape)
 cudaError_t launch_warp(int E, const WarpArgs &a, int warps_per_block,
                         int grid, size_t smem, cudaStream_t st);
-cudaError_t warp_set_smem(int E, size_t smem);
-cudaError_t warp_occupancy(int E, int warps_per_block, size_t smem, int *blocks);
+// occupancies of the kernel a launch at Lc lanes per cell with those tickets
+// (tk) runs
+cudaError_t warp_occupancy(int E, int Lc, int tk, int warps_per_block, size_t smem, int *blocks);
 // persistent batch kernel: E in {3,4,5,6,8}, A staged in shared memory or not
 const void *batch_kernel(int E, bool a_smem);
 cudaError_t batch_prepare(int E, bool a_smem, int warps_per_block, size_t smem,
@@ -178,11 +199,11 @@ cudaError_t block_set_smem(size_t smem);
 // fused-assembly solve, E in 1..8
 cudaError_t launch_assemble(int E, const WarpArgs &a, int warps_per_block,
                             int grid, size_t smem, cudaStream_t st);
-cudaError_t assemble_occupancy(int E, int warps_per_block, size_t smem, int *blocks);
+cudaError_t assemble_occupancy(int E, int Lc, int tk, int warps_per_block, size_t smem, int *blocks);
 // device Newton corrector around the fused assembly + solve, E in 1..8
 cudaError_t launch_newton(int E, const WarpArgs &a, int warps_per_block,
                           int grid, size_t smem, cudaStream_t st);
-cudaError_t newton_occupancy(int E, int warps_per_block, size_t smem, int *blocks);
+cudaError_t newton_occupancy(int E, int Lc, int tk, int warps_per_block, size_t smem, int *blocks);
 cudaError_t launch_grad(const GradArgs &a, cudaStream_t st);
 // Difficulty ordering: cells binned by decreasing max_i |A_ii - 1| (half
 // octaves), written to *order (inside the caller's scratch of
@@ -211,6 +232,13 @@ const void *batch_classify_kernel_fn();  // __global__ (const BatchOrderArgs)
 const void *batch_scatter_kernel_fn();   // __global__ (const BatchOrderArgs), 1 thread per cell
 
 constexpr int kMaxE = 16;  // rows per lane supported by the warp kernel
+// Tickets of a plain launch: groups of k cells, single cells, or groups and
+// then single cells (the last two at 16 lanes per cell).
+constexpr int kTicketsPack = 0, kTicketsOne = 1, kTicketsBoth = 2;
+inline int tickets_of(const WarpArgs &a) {
+  if (!a.sched2 || a.single_from >= a.ngroups) return kTicketsPack;
+  return a.single_from == 0 ? kTicketsOne : kTicketsBoth;
+}
 
 // Difficulty classes of the ordering (half octaves of max_i |A_ii - 1|) and
 // the in-launch ordering's workspace: class totals, one barrier counter
@@ -264,9 +292,12 @@ struct MixedArgs {
   int *status;    // or null
   const SchedWord *sched;
   const int *src;
-  const int *dst;
-  const int *padfrom;
-  const int *dslot;
+  const int *dst;      // [nnz] place (pair_pos) of each A entry in the FP64 copy
+  const int *dst32;    // [nnz] place (word_pos) of each A entry in the FP32 copy
+  const int *pads, *pads32;  // [npads] places of the padding slots in either copy
+  int npads;
+  unsigned ends[kEndWords];
+  const int *dslot32;  // [n] place (word_pos) of each row's diagonal entry
   double tol;
   int max_sweeps;
   float tol_in;
@@ -285,6 +316,11 @@ struct MixedArgs {
   int *ord_err;
   long long ord_wait;
 };
+// Shared-memory bytes per cell of the refinement kernel: FP32 A, FP64 A when
+// staged, two FP64 and three FP32 vectors, rounded to 16.
+__host__ __device__ inline size_t mixed_cell_bytes(int segA, int segV, bool a64_smem) {
+  return ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)28 * segV + 15) & ~(size_t)15;
+}
 // a cooperative launch when a.ord_ws is set (grid at most SMs x occupancy)
 cudaError_t launch_mixed(int E, const MixedArgs &a, int warps_per_block,
                          int grid, size_t smem, cudaStream_t st);

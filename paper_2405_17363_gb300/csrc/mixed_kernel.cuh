@@ -32,7 +32,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
   const int n = a.n, nnz = a.nnz;
   // bytes per cell: (12 or 4) segA + 16 segV + 12 segV (FP64 A when staged,
   // FP32 A, 2 FP64 + 3 FP32 vectors)
-  const size_t cellBytes = (size_t)(a.a64_smem ? 12 : 4) * a.segA + (size_t)28 * a.segV;
+  const size_t cellBytes = mixed_cell_bytes(a.segA, a.segV, a.a64_smem);
   unsigned char *wb = smem_raw + sched_smem_bytes(nsch) +
                       ((size_t)warp * a.k + seg) * cellBytes;
   double *As = reinterpret_cast<double *>(wb);
@@ -50,7 +50,9 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
     g64[i] = 0.0; o64[i] = 0.0; g32[i] = 0.0f; o1[i] = 0.0f; o2[i] = 0.0f;
   }
   __syncthreads();
-  const SchedWord *sch = sch_s + sl;
+  const SchedWord *sch = sch_s;
+  const unsigned g64a = smem_addr(g64), o64a = smem_addr(o64), g32a = smem_addr(g32),
+                 o1a = smem_addr(o1), o2a = smem_addr(o2);
   const int warps_total = gridDim.x * (blockDim.x >> 5);
   constexpr int K = LC ? 32 / LC : 0;  // cells per warp (0: a.k)
 
@@ -65,15 +67,11 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
                       : pos;
     const double *Ac = a.A + (size_t)(has ? c : 0) * nnz;
     if (a.a64_smem) {  // stage A in slot order, FP64 and its FP32 rounding
-      stage_scatter(Ac, a.dst, nnz, sl, Lc, has, [&](int t, double v) {
-        As[t] = v;
-        As32[t] = d2f_rn(v);
-      });
-      zero_padding(As, a.padfrom, a.L, Lc, sl);
-    } else {  // the FP32 rounding only
-      stage_scatter(Ac, a.dst, nnz, sl, Lc, has, [&](int t, double v) { As32[t] = d2f_rn(v); });
+      stage_scatter(Ac, a.dst, nnz, sl, Lc, has, [&](int t, double v) { As[t] = v; });
+      zero_padding(As, a.pads, a.npads, a.L, sl, Lc);
     }
-    zero_padding(As32, a.padfrom, a.L, Lc, sl);
+    stage_scatter(Ac, a.dst32, nnz, sl, Lc, has, [&](int t, double v) { As32[t] = d2f_rn(v); });
+    zero_padding(As32, a.pads32, a.npads, a.L, sl, Lc);
     __syncwarp();
     double xv[E];
     float dinv[E];
@@ -85,7 +83,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
         const int i = sl + e * Lc;
         const bool v = has && i < n;
         const double bi = v ? __ldg(a.b + (size_t)c * n + i) : 0.0;
-        const float d = v ? As32[__ldg(a.dslot + i)] : 0.0f;
+        const float d = v ? As32[__ldg(a.dslot32 + i)] : 0.0f;
         dinv[e] = v ? (d != 0.0f ? 1.0f / d : 1.0f) : 0.0f;
         xv[e] = 0.0;
         acc[0] = fma(bi, bi, acc[0]);
@@ -111,8 +109,8 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 #pragma unroll
         for (int e = 0; e < E; ++e) g64[sl + e * Lc] = xv[e];
         __syncwarp();
-        if (a.a64_smem) seg_spmv(sch, a.L, Lc, As + sl, g64, o64);
-        else seg_spmv_gather(sch, a.src + sl, a.L, Lc, Ac, g64, o64);
+        if (a.a64_smem) seg_spmv(sch, a.ends, a.L, Lc, sl, As, g64a, o64a);
+        else seg_spmv_gather(sch, a.ends, a.src, a.L, Lc, sl, Ac, g64a, o64a);
         __syncwarp();
       }
       double rr[1] = {0.0};
@@ -154,7 +152,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
       }
       const double rn64 = wide ? sqrt(rr[0]) : 0.0;
       const double sc64 = wide ? 1.0 / rn64 : 0.0;
-      float rf[E], rh[E], p[E], s[E], d[E];
+      float rf[E], rh[E], p[E], d[E];  // rf also holds s = r - alpha v
       float cc[1] = {0.0f};
 #pragma unroll
       for (int e = 0; e < E; ++e) {
@@ -162,7 +160,6 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
         rf[e] = ce;
         rh[e] = ce;
         p[e] = 0.0f;
-        s[e] = 0.0f;
         d[e] = 0.0f;
         cc[0] = fmaf(ce, ce, cc[0]);
       }
@@ -171,18 +168,26 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
       float rho = cc[0], rho_prev = 1.0f, alpha = 1.0f, omega = 1.0f;
       bool act = !done && cc[0] > 0.0f && isfinite(cc[0]);
       int it = 0;
+      bool head = true;  // first iteration: p = r
       while (__any_sync(kFull, act)) {
         if (act) {
           if (it >= a.maxit_in || !isfinite(rho) || fabsf(rho) < 1e-37f) act = false;
         }
-        const float beta = (rho / rho_prev) * (alpha / omega);
+        // p = r + beta (p - omega v), v of the iteration before
+        if (head) {
+          head = false;
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-          if (act) p[e] = fmaf(beta, p[e], rf[e]);
-          g32[sl + e * Lc] = dinv[e] * p[e];
+          for (int e = 0; e < E; ++e) p[e] = rf[e];
+        } else {
+          const float beta = (rho / rho_prev) * (alpha / omega);
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+            p[e] = fmaf(beta, fmaf(-omega, o1[sl + e * Lc], p[e]), rf[e]);
         }
+#pragma unroll
+        for (int e = 0; e < E; ++e) g32[sl + e * Lc] = dinv[e] * p[e];
         __syncwarp();
-        seg_spmvf(sch, a.L, Lc, As32 + sl, g32, o1);
+        seg_spmvf(sch, a.L, Lc, sl, As32, g32a, o1a);
         __syncwarp();
         if (act) ++it;
         float sg[1] = {0.0f};
@@ -190,46 +195,45 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
         for (int e = 0; e < E; ++e) sg[0] = fmaf(rh[e], o1[sl + e * Lc], sg[0]);
         seg_sumf<1>(sg, Lc);
         if (act && (!isfinite(sg[0]) || fabsf(sg[0]) < 1e-37f)) act = false;
-        const float al = rho / sg[0];
-        if (act) alpha = al;
+        alpha = rho / sg[0];
+        float q0[1] = {0.0f};
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const int i = sl + e * Lc;
-          if (act) {
-            d[e] = fmaf(al, g32[i], d[e]);
-            s[e] = fmaf(-al, o1[i], rf[e]);
-          }
-          g32[i] = dinv[e] * s[e];
+          if (act) d[e] = fmaf(alpha, g32[i], d[e]);
+          rf[e] = fmaf(-alpha, o1[i], rf[e]);  // s
+          q0[0] = fmaf(rf[e], rf[e], q0[0]);
         }
+        seg_sumf<1>(q0, Lc);
+        // converged on the half step: tested before the second product
+        if (act && q0[0] <= thr) act = false;
+        if (!__any_sync(kFull, act)) break;
+#pragma unroll
+        for (int e = 0; e < E; ++e) g32[sl + e * Lc] = dinv[e] * rf[e];
         __syncwarp();
-        seg_spmvf(sch, a.L, Lc, As32 + sl, g32, o2);
+        seg_spmvf(sch, a.L, Lc, sl, As32, g32a, o2a);
         __syncwarp();
-        float q3[3] = {0.0f, 0.0f, 0.0f};
+        float qt[2] = {0.0f, 0.0f};
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const float t = o2[sl + e * Lc];
-          q3[0] = fmaf(s[e], s[e], q3[0]);
-          q3[1] = fmaf(t, s[e], q3[1]);
-          q3[2] = fmaf(t, t, q3[2]);
+          qt[0] = fmaf(t, rf[e], qt[0]);
+          qt[1] = fmaf(t, t, qt[1]);
         }
-        seg_sumf<3>(q3, Lc);
+        seg_sumf<2>(qt, Lc);
         bool full = false;
         if (act) {
-          if (q3[0] <= thr || !isfinite(q3[1]) || !isfinite(q3[2]) || q3[2] == 0.0f)
+          if (!isfinite(qt[0]) || !isfinite(qt[1]) || qt[1] == 0.0f)
             act = false;
           else
             full = true;
         }
-        const float om = q3[1] / q3[2];
-        if (full) omega = om;
+        omega = qt[0] / qt[1];
 #pragma unroll
         for (int e = 0; e < E; ++e) {
           const int i = sl + e * Lc;
-          if (full) {
-            d[e] = fmaf(om, g32[i], d[e]);
-            rf[e] = fmaf(-om, o2[i], s[e]);
-            p[e] = fmaf(-om, o1[i], p[e]);
-          }
+          if (full) d[e] = fmaf(omega, g32[i], d[e]);
+          rf[e] = fmaf(-omega, o2[i], rf[e]);
         }
         float q2[2] = {0.0f, 0.0f};
 #pragma unroll
@@ -239,13 +243,10 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
         }
         seg_sumf<2>(q2, Lc);
         if (full) {
-          if (q2[1] <= thr || om == 0.0f) {
-            act = false;
-          } else {
-            rho_prev = rho;
-            rho = q2[0];
-          }
+          if (q2[1] <= thr || omega == 0.0f) act = false;
         }
+        rho_prev = rho;
+        rho = q2[0];
       }
       if (!done) {
         inner += it;
@@ -289,7 +290,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 }
 
 template <int E>
-__global__ void __launch_bounds__(256, 2) mixed_refine_kernel(const MixedArgs a) {
+__global__ void __launch_bounds__(256, 2) mixed_refine_kernel(const __grid_constant__ MixedArgs a) {
   // the automatic choice (at most 3 rows per lane on 8, 16 or 32 lanes) runs
   // code with the lane count fixed at compile time
   if constexpr (E >= 2 && E <= 3) {

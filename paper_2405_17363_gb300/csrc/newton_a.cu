@@ -3,8 +3,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 1)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 2)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 3)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 4)
+CAMP_KERNEL_DEFINE(newton, 1)
+CAMP_KERNEL_DEFINE(newton, 2)
+CAMP_KERNEL_DEFINE(newton, 3)
+CAMP_KERNEL_DEFINE(newton, 4)
 }  // namespace camp

@@ -3,8 +3,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 5)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 6)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 7)
-CAMP_KERNEL_DEFINE(newton, newton_bicgstab_kernel, 8)
+CAMP_KERNEL_DEFINE(newton, 5)
+CAMP_KERNEL_DEFINE(newton, 6)
+CAMP_KERNEL_DEFINE(newton, 7)
+CAMP_KERNEL_DEFINE(newton, 8)
 }  // namespace camp

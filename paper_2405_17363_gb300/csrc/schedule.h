@@ -23,9 +23,31 @@
 // conflict-free.
 #pragma once
 #include <stddef.h>
+#include "camp_internal.h"
 
 namespace camp {
 namespace sched {
+
+constexpr unsigned kEnd = 0x80000000u;  // host slot word: last slot of a row
+
+// Host slot words ([slot][lane]: column | row << 11 | end << 31) to the
+// device words at their word_pos places.
+inline void pack_words(int L, int Lc, const unsigned *word, SchedWord *out) {
+  for (int j = 0; j < L; ++j)
+    for (int q = 0; q < Lc; ++q) {
+      const unsigned w = word[(size_t)j * Lc + q];
+      out[word_pos(j, q, L, Lc)] =
+          slot_word((int)(w & 0x7ffu), (int)((w >> 11) & 0x7ffu), (w & kEnd) != 0u);
+    }
+}
+
+// ends: bit j % 32 of word j / 32 set when some lane ends a row in slot j.
+inline void end_mask(int L, int Lc, const unsigned *word, unsigned *ends) {
+  for (int i = 0; i < kEndWords; ++i) ends[i] = 0u;
+  for (int j = 0; j < L && j < 32 * kEndWords; ++j)
+    for (int q = 0; q < Lc; ++q)
+      if (word[(size_t)j * Lc + q] & kEnd) ends[j >> 5] |= 1u << (j & 31);
+}
 
 // Work buffers of build (caller-owned; sizes in elements).
 struct Work {

@@ -14,17 +14,16 @@
 
 #include "camp_internal.h"
 #include "camp_testing.h"
+#include "align.h"
 #include "schedule.h"
 
 namespace camp {
-cudaError_t launch_warp_1(const WarpArgs &, int, int, size_t, cudaStream_t);
 #define CAMP_DECL(E)                                                        \
   cudaError_t launch_warp_##E(const WarpArgs &, int, int, size_t, cudaStream_t); \
-  cudaError_t occ_warp_##E(int, size_t, int *);
-CAMP_DECL(2) CAMP_DECL(3) CAMP_DECL(4) CAMP_DECL(5) CAMP_DECL(6) CAMP_DECL(7)
+  cudaError_t occ_warp_##E(int, int, int, size_t, int *);
+CAMP_DECL(1) CAMP_DECL(2) CAMP_DECL(3) CAMP_DECL(4) CAMP_DECL(5) CAMP_DECL(6) CAMP_DECL(7)
 CAMP_DECL(8) CAMP_DECL(9) CAMP_DECL(10) CAMP_DECL(11) CAMP_DECL(12)
 CAMP_DECL(13) CAMP_DECL(14) CAMP_DECL(15) CAMP_DECL(16)
-cudaError_t occ_warp_1(int, size_t, int *);
 #define CAMP_DECLM(E)                                                        \
   cudaError_t launch_mixed_##E(const MixedArgs &, int, int, size_t, cudaStream_t); \
   cudaError_t occ_mixed_##E(int, size_t, int *);
@@ -34,9 +33,9 @@ CAMP_DECLM(11) CAMP_DECLM(12) CAMP_DECLM(13) CAMP_DECLM(14) CAMP_DECLM(15)
 CAMP_DECLM(16)
 #define CAMP_DECLF(E)                                                         \
   cudaError_t launch_assemble_##E(const WarpArgs &, int, int, size_t, cudaStream_t); \
-  cudaError_t occ_assemble_##E(int, size_t, int *);                            \
+  cudaError_t occ_assemble_##E(int, int, int, size_t, int *);                  \
   cudaError_t launch_newton_##E(const WarpArgs &, int, int, size_t, cudaStream_t);   \
-  cudaError_t occ_newton_##E(int, size_t, int *);
+  cudaError_t occ_newton_##E(int, int, int, size_t, int *);
 CAMP_DECLF(1) CAMP_DECLF(2) CAMP_DECLF(3) CAMP_DECLF(4) CAMP_DECLF(5)
 CAMP_DECLF(6) CAMP_DECLF(7) CAMP_DECLF(8)
 #undef CAMP_DECLF
@@ -53,9 +52,9 @@ cudaError_t launch_warp(int E, const WarpArgs &a, int wpb, int grid,
     default: return cudaErrorInvalidValue;
   }
 }
-static cudaError_t warp_occupancy_query(int E, int wpb, size_t smem, int *blocks) {
+static cudaError_t warp_occupancy_query(int E, int Lc, int tk, int wpb, size_t smem, int *blocks) {
   switch (E) {
-#define C(E) case E: return occ_warp_##E(wpb, smem, blocks);
+#define C(E) case E: return occ_warp_##E(Lc, tk, wpb, smem, blocks);
     C(1) C(2) C(3) C(4) C(5) C(6) C(7) C(8) C(9) C(10) C(11) C(12) C(13)
     C(14) C(15) C(16)
 #undef C
@@ -65,8 +64,8 @@ static cudaError_t warp_occupancy_query(int E, int wpb, size_t smem, int *blocks
 
 // The occupancy of a launch shape does not change: remember the answers
 // (fixed-size record, no heap allocation).
-cudaError_t warp_occupancy(int E, int wpb, size_t smem, int *blocks) {
-  struct Entry { int dev, E, wpb; size_t smem; int blocks; };
+cudaError_t warp_occupancy(int E, int Lc, int tk, int wpb, size_t smem, int *blocks) {
+  struct Entry { int dev, E, Lc, tk, wpb; size_t smem; int blocks; };
   static std::mutex mu;
   static Entry memo[256];
   static int nmemo = 0;
@@ -76,14 +75,15 @@ cudaError_t warp_occupancy(int E, int wpb, size_t smem, int *blocks) {
   {
     std::lock_guard<std::mutex> lock(mu);
     for (int i = 0; i < nmemo; ++i)
-      if (memo[i].dev == dev && memo[i].E == E && memo[i].wpb == wpb && memo[i].smem == smem) {
+      if (memo[i].dev == dev && memo[i].E == E && memo[i].Lc == Lc && memo[i].tk == tk &&
+          memo[i].wpb == wpb && memo[i].smem == smem) {
         *blocks = memo[i].blocks;
         return cudaSuccess;
       }
   }
-  if ((e = warp_occupancy_query(E, wpb, smem, blocks)) != cudaSuccess) return e;
+  if ((e = warp_occupancy_query(E, Lc, tk, wpb, smem, blocks)) != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mu);
-  if (nmemo < 256) memo[nmemo++] = Entry{dev, E, wpb, smem, *blocks};
+  if (nmemo < 256) memo[nmemo++] = Entry{dev, E, Lc, tk, wpb, smem, *blocks};
   return cudaSuccess;
 }
 
@@ -123,16 +123,16 @@ cudaError_t mixed_occupancy(int E, int wpb, size_t smem, int *blocks) {
     }                                                                           \
   }
 #define CAMP_OCCUPANCY8(fn, name)                                             \
-  cudaError_t fn(int E, int wpb, size_t smem, int *blocks) {                    \
+  cudaError_t fn(int E, int Lc, int tk, int wpb, size_t smem, int *blocks) {    \
     switch (E) {                                                                \
-      case 1: return occ_##name##_1(wpb, smem, blocks);                         \
-      case 2: return occ_##name##_2(wpb, smem, blocks);                         \
-      case 3: return occ_##name##_3(wpb, smem, blocks);                         \
-      case 4: return occ_##name##_4(wpb, smem, blocks);                         \
-      case 5: return occ_##name##_5(wpb, smem, blocks);                         \
-      case 6: return occ_##name##_6(wpb, smem, blocks);                         \
-      case 7: return occ_##name##_7(wpb, smem, blocks);                         \
-      case 8: return occ_##name##_8(wpb, smem, blocks);                         \
+      case 1: return occ_##name##_1(Lc, tk, wpb, smem, blocks);                 \
+      case 2: return occ_##name##_2(Lc, tk, wpb, smem, blocks);                 \
+      case 3: return occ_##name##_3(Lc, tk, wpb, smem, blocks);                 \
+      case 4: return occ_##name##_4(Lc, tk, wpb, smem, blocks);                 \
+      case 5: return occ_##name##_5(Lc, tk, wpb, smem, blocks);                 \
+      case 6: return occ_##name##_6(Lc, tk, wpb, smem, blocks);                 \
+      case 7: return occ_##name##_7(Lc, tk, wpb, smem, blocks);                 \
+      case 8: return occ_##name##_8(Lc, tk, wpb, smem, blocks);                 \
       default: return cudaErrorInvalidValue;                                    \
     }                                                                           \
   }
@@ -198,23 +198,17 @@ camp_status cuda_fail(cudaError_t e, const char *where) {
 // and for every row the slot of its diagonal entry.
 struct Schedule {
   int Lc = 0, L = 0;
-  std::vector<SchedWord> words;  // [L][Lc]
+  // slot t = j * Lc + lane: the words of sched::build
+  std::vector<unsigned> words;   // [L][Lc]
   std::vector<int> src;          // [L][Lc], -1 = padding
   std::vector<int> dslot;        // [n]
   std::vector<int> dst;          // [nnz] slot of each A entry (forward order)
   std::vector<int> padfrom;      // [Lc] first padding slot of each lane
-  // automatic warps per block, found once per kernel kind (0: not yet):
-  // plain solve, fused assembly, Newton corrector
-  int auto_wpb[3] = {0, 0, 0};
-  SchedWord *d_words = nullptr;
-  int *d_src = nullptr, *d_dslot = nullptr, *d_dst = nullptr, *d_padfrom = nullptr;
   // 16 lanes per cell only: the split schedule of one cell on 32 lanes (L2
   // 0: none); see split_schedule
   int L2 = 0;
-  std::vector<SchedWord> words2;  // [L2][32]
+  std::vector<unsigned> words2;  // [L2][32]
   std::vector<int> dst2, padfrom2, dslot2;
-  SchedWord *d_words2 = nullptr;
-  int *d_dst2 = nullptr, *d_padfrom2 = nullptr, *d_dslot2 = nullptr;
 };
 
 // The split schedule of a 16-lane schedule: one cell on all 32 lanes, lane v
@@ -233,7 +227,7 @@ void split_schedule(Schedule &S, int n, int nnz) {
   for (int v = 0; v < 16; ++v) {
     const int len = S.padfrom[v];
     for (int j = 0, st = 0; j < len; ++j)
-      if (S.words[(size_t)j * 16 + v] & kSlotEnd) {
+      if (S.words[(size_t)j * 16 + v] & sched::kEnd) {
         rstart[v].push_back(st);
         rlen[v].push_back(j + 1 - st);
         st = j + 1;
@@ -308,7 +302,7 @@ Schedule build_schedule(int n, const std::vector<int> &rp,
                          cursor.data(), cur_row.data(), rem.data(), rem_count.data()};
   long total = 0;  // an upper bound of L * Lc: every row on one lane
   for (int r = 0; r < n; ++r) total += rp[r + 1] - rp[r];
-  std::vector<SchedWord> words((size_t)total * Lc);
+  std::vector<unsigned> words((size_t)total * Lc);
   std::vector<int> entry((size_t)total * Lc);
   Schedule S;
   S.Lc = Lc;
@@ -328,12 +322,45 @@ Schedule build_schedule(int n, const std::vector<int> &rp,
   return S;
 }
 
+// A schedule as the kernels run it: slots by lane (word_pos and pair_pos
+// places, camp_internal.h), on the device.
+struct Slots {
+  int Lc = 0, L = 0, npads = 0;
+  std::vector<int> dst;      // [nnz] slot (j * Lc + lane) of each A entry
+  unsigned ends[kEndWords] = {};
+  SchedWord *d_words = nullptr;
+  int *d_src = nullptr;      // word_pos places
+  int *d_dst = nullptr, *d_dslot = nullptr, *d_pads = nullptr;        // pair_pos places
+  int *d_dst32 = nullptr, *d_dslot32 = nullptr, *d_pads32 = nullptr;  // word_pos places
+  int *d_dentry = nullptr;   // [n] A entry of each row's diagonal
+  void release() {
+    for (void *p : {(void *)d_words, (void *)d_src, (void *)d_dst, (void *)d_dslot,
+                    (void *)d_pads, (void *)d_dst32, (void *)d_dslot32, (void *)d_pads32,
+                    (void *)d_dentry})
+      cudaFree(p);
+  }
+};
+
+// The layouts of one lane count, each built when first used (L 0: not yet).
+enum Kind {
+  kPlain = 0,    // the schedule as built (the refinement kernel)
+  kAligned = 1,  // its rows aligned (align.h), where that takes no more slots
+  kOne = 2,      // at 16 lanes: the cell alone on 32 lanes
+};
+struct Layout {
+  Schedule base;
+  Slots slots[3];
+  // automatic warps per block, found once per kernel kind (0: not yet):
+  // plain solve, fused assembly, Newton corrector
+  int auto_wpb[3] = {0, 0, 0};
+};
+
 // one orientation of the pattern: forward (A) or transposed (A^T)
 struct View {
   int n = 0, nnz = 0;
   std::vector<int> rp, ci, diag, perm;  // perm empty for the forward view
   int *d_rp = nullptr, *d_ci = nullptr, *d_diag = nullptr, *d_perm = nullptr;
-  std::map<int, Schedule> sched;  // by lanes per cell
+  std::map<int, Layout> sched;  // by lanes per cell
 };
 
 template <class T>
@@ -431,36 +458,108 @@ struct camp_solver {
 
 namespace {
 
-cudaError_t view_schedule(View &v, int Lc, Schedule **out) {
+// The device form of the slots word/src [L][Lc] (host words, A entry or -1);
+// dentry: the A entry of every row's diagonal.
+cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<unsigned> &word,
+                         const std::vector<int> &src, const std::vector<int> &dentry) {
+  S.Lc = Lc;
+  S.L = L;
+  S.dst.assign(nnz, -1);
+  std::vector<SchedWord> words((size_t)L * Lc);
+  sched::pack_words(L, Lc, word.data(), words.data());
+  sched::end_mask(L, Lc, word.data(), S.ends);
+  std::vector<int> psrc((size_t)L * Lc), dst(nnz, -1), dst32(nnz, -1), pads, pads32;
+  for (int j = 0; j < L; ++j)
+    for (int q = 0; q < Lc; ++q) {
+      const int k = src[(size_t)j * Lc + q];
+      const int pp = pair_pos(j, q, L, Lc), wp = word_pos(j, q, L, Lc);
+      psrc[wp] = k;
+      if (k < 0) {
+        pads.push_back(pp);
+        pads32.push_back(wp);
+        continue;
+      }
+      S.dst[k] = j * Lc + q;
+      dst[k] = pp;
+      dst32[k] = wp;
+    }
+  S.npads = (int)pads.size();
+  std::vector<int> dslot(dentry.size()), dslot32(dentry.size());
+  for (size_t i = 0; i < dentry.size(); ++i) {
+    dslot[i] = dst[dentry[i]];
+    dslot32[i] = dst32[dentry[i]];
+  }
+  cudaError_t e = upload(&S.d_words, words);
+  if (e == cudaSuccess) e = upload(&S.d_src, psrc);
+  if (e == cudaSuccess) e = upload(&S.d_dst, dst);
+  if (e == cudaSuccess) e = upload(&S.d_dslot, dslot);
+  if (e == cudaSuccess) e = upload(&S.d_pads, pads);
+  if (e == cudaSuccess) e = upload(&S.d_dst32, dst32);
+  if (e == cudaSuccess) e = upload(&S.d_dslot32, dslot32);
+  if (e == cudaSuccess) e = upload(&S.d_pads32, pads32);
+  if (e == cudaSuccess) e = upload(&S.d_dentry, dentry);
+  return e;
+}
+
+// Every row's entries in the order of the schedule S.
+sched::RowChains row_chains(const Schedule &S, const std::vector<int> &rp) {
+  const int n = (int)rp.size() - 1;
+  sched::RowChains ch;
+  ch.start = rp;
+  ch.entry.resize(rp[n]);
+  ch.col.resize(rp[n]);
+  std::vector<int> fill(rp.begin(), rp.end() - 1);
+  for (int q = 0; q < S.Lc; ++q)
+    for (int j = 0; j < S.L; ++j) {
+      const size_t t = (size_t)j * S.Lc + q;
+      if (S.src[t] < 0) continue;
+      const int k = fill[(S.words[t] >> 11) & 0x7ffu]++;
+      ch.entry[k] = S.src[t];
+      ch.col[k] = (int)(S.words[t] & 0x7ffu);
+    }
+  return ch;
+}
+
+// A layout of the view's rows at Lc lanes per cell.  Every row keeps the
+// entry order of its Lc-lane schedule in each, so its sum keeps its bits.
+cudaError_t view_schedule(View &v, int Lc, Kind kind, Layout **out, const Slots **slots) {
   auto it = v.sched.find(Lc);
   if (it == v.sched.end()) {
-    Schedule S = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
-    split_schedule(S, v.n, v.nnz);
-    cudaError_t e = upload(&S.d_words, S.words);
-    if (e == cudaSuccess) e = upload(&S.d_src, S.src);
-    if (e == cudaSuccess) e = upload(&S.d_dslot, S.dslot);
-    if (e == cudaSuccess) e = upload(&S.d_dst, S.dst);
-    if (e == cudaSuccess) e = upload(&S.d_padfrom, S.padfrom);
-    if (e == cudaSuccess && S.L2) e = upload(&S.d_words2, S.words2);
-    if (e == cudaSuccess && S.L2) e = upload(&S.d_dst2, S.dst2);
-    if (e == cudaSuccess && S.L2) e = upload(&S.d_padfrom2, S.padfrom2);
-    if (e == cudaSuccess && S.L2) e = upload(&S.d_dslot2, S.dslot2);
-    if (e != cudaSuccess) {
-      cudaFree(S.d_words);
-      cudaFree(S.d_src);
-      cudaFree(S.d_dslot);
-      cudaFree(S.d_dst);
-      cudaFree(S.d_padfrom);
-      cudaFree(S.d_words2);
-      cudaFree(S.d_dst2);
-      cudaFree(S.d_padfrom2);
-      cudaFree(S.d_dslot2);
-      return e;
-    }
-    it = v.sched.emplace(Lc, std::move(S)).first;
+    it = v.sched.emplace(Lc, Layout()).first;
+    it->second.base = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
   }
-  *out = &it->second;
-  return cudaSuccess;
+  Layout &Y = it->second;
+  Slots &to = Y.slots[kind];
+  if (out) *out = &Y;
+  *slots = &to;
+  if (to.L) return cudaSuccess;
+  Schedule &S = Y.base;
+  std::vector<int> dentry(v.n);
+  for (int i = 0; i < v.n; ++i) dentry[i] = S.src[S.dslot[i]];
+  std::vector<unsigned> word;
+  std::vector<int> src;
+  int L = 0;
+  const int lanes = kind == kOne ? 32 : Lc;
+  if (kind != kPlain) {
+    if (kind == kOne) split_schedule(S, v.n, v.nnz);
+    L = sched::align(v.n, row_chains(S, v.rp), lanes, kind == kOne ? S.L2 : S.L, word, src);
+  }
+  if (L == 0 && kind == kOne) {
+    L = S.L2;
+    word = S.words2;
+    src.assign(word.size(), -1);
+    for (int k = 0; k < v.nnz; ++k) src[S.dst2[k]] = k;
+  } else if (L == 0) {
+    L = S.L;
+    word = S.words;
+    src = S.src;
+  }
+  const cudaError_t e = upload_slots(to, lanes, L, v.nnz, word, src, dentry);
+  if (e != cudaSuccess) {
+    to.release();
+    to = Slots();
+  }
+  return e;
 }
 
 void free_view(View &v) {
@@ -468,18 +567,21 @@ void free_view(View &v) {
   cudaFree(v.d_ci);
   cudaFree(v.d_diag);
   cudaFree(v.d_perm);
-  for (auto &kv : v.sched) {
-    cudaFree(kv.second.d_words);
-    cudaFree(kv.second.d_src);
-    cudaFree(kv.second.d_dslot);
-    cudaFree(kv.second.d_dst);
-    cudaFree(kv.second.d_padfrom);
-    cudaFree(kv.second.d_words2);
-    cudaFree(kv.second.d_dst2);
-    cudaFree(kv.second.d_padfrom2);
-    cudaFree(kv.second.d_dslot2);
-  }
+  for (auto &kv : v.sched)
+    for (Slots &S : kv.second.slots) S.release();
   v.sched.clear();
+}
+
+// A launch's schedule arguments.
+template <class Args>
+void set_slots(Args &a, const Slots &S) {
+  a.L = S.L;
+  a.sched = S.d_words;
+  a.src = S.d_src;
+  a.dst = S.d_dst;
+  a.pads = S.d_pads;
+  a.npads = S.npads;
+  memcpy(a.ends, S.ends, sizeof a.ends);
 }
 
 int ilog2(int v) {
@@ -496,7 +598,7 @@ int ilog2(int v) {
 // schedule's gathers (columns of distinct residues modulo Lc, schedule.h)
 // stay conflict-free.
 int bank_spread_stride(int need, int k) {
-  const int want = (32 / k) % 16;
+  const int want = k == 32 ? 2 : (32 / k) % 16;  // even: a cell's block starts at 16 bytes
   int s = need;
   while (s % 16 != want) ++s;
   return s;
@@ -518,7 +620,7 @@ size_t warp_smem(const View &v, int Lc, int L, int wpb, int *segA, int *segV,
 // warps per SM (the CTA's schedule copy and its warps' cell regions must pack
 // into the SM's shared memory; occ gives the CTAs per SM of the kernel), 4
 // unless another count fits more.  Fills the shared-memory layout.
-typedef cudaError_t (*OccFn)(int E, int wpb, size_t smem, int *blocks);
+typedef cudaError_t (*OccFn)(int E, int Lc, int tk, int wpb, size_t smem, int *blocks);
 cudaError_t pick_warps_per_block(const View &v, int Lc, int L, int E, int extra_vectors,
                                  size_t optin, OccFn occ_fn, int *cache, int *wpb, size_t *smem,
                                  int *segA, int *segV, int *segStride) {
@@ -532,7 +634,7 @@ cudaError_t pick_warps_per_block(const View &v, int Lc, int L, int E, int extra_
     int sa = 0, sv = 0, ss = 0, occ = 0;
     const size_t sm = warp_smem(v, Lc, L, w, &sa, &sv, &ss, extra_vectors);
     if (sm > optin) continue;
-    const cudaError_t e = occ_fn(E, w, sm, &occ);
+    const cudaError_t e = occ_fn(E, Lc, kTicketsPack, w, sm, &occ);
     if (e != cudaSuccess) return e;
     if (occ * w > best) {
       best = occ * w;
@@ -552,9 +654,9 @@ size_t mixed_smem(const View &v, int Lc, int L, int wpb, int *segA, int *segV, b
   const int k = 32 / Lc;
   const int E = (v.n + Lc - 1) / Lc;
   *segA = (L * Lc + 1) & ~1;  // A in slot order
-  *segV = ((E * Lc + 1) + 1) & ~1;
+  *segV = (E * Lc + 1) & ~1;
   const size_t sch = sched_smem_bytes(L * Lc);
-  return sch + (size_t)wpb * k * ((size_t)(a64_smem ? 12 : 4) * *segA + (size_t)28 * *segV);
+  return sch + (size_t)wpb * k * mixed_cell_bytes(*segA, *segV, a64_smem);
 }
 
 // Automatic arrangement: the most cells per warp (fewest lanes per cell) that
@@ -816,40 +918,48 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 
 // Single-cell tickets of a plain launch at 16 lanes per cell (warp_single.cuh):
 // the last R pairs of the launch become 2R single-cell tickets.  Automatic R
-// (measured at 80 species on 152 SMs x 16 warps): every pair when the pairs
-// would keep at most a quarter of the resident warps busy (a lone warp's
-// latency decides such a launch: 60 against 75 us at 64 to 608 cells, 65.5
-// against 75.8 at 1,212), else none (at full load one cell per warp costs
-// about 13 % more per cell, and turning the pairs past the last full wave
-// into singles measured within the noise at 10,000 cells).
+// (measured at 80 species on 152 SMs x 12 warps): every pair when the pairs
+// would keep at most three quarters of the resident warps busy (a lone warp's
+// latency decides such a launch: 49 against 62 us at 600 cells, 81 against 86
+// at 3,000, 108 against 91 at 4,000), a third when the launch shares the GPU
+// with others (`shared`: the chunks of the host-memory pipeline), else none
+// (at full load one cell per warp costs about 13 % more per cell).
 // camp_solver_set_single_tail overrides it.  Sets
 // single_from, ngroups (tickets) and the split schedule's arguments; leaves
 // the launch without single tickets when the split schedule does not fit
 // the warp's region.
-void set_single_tickets(camp_solver_t h, const Schedule &S, WarpArgs &a, int wpb, int occ) {
+cudaError_t set_single_tickets(camp_solver_t h, View &v, WarpArgs &a, int wpb, int occ,
+                               bool shared) {
   const int pairs = a.ngroups;
   a.single_from = pairs;
   a.sched2 = nullptr;
-  if (S.L2 == 0 || a.Lc != 16 || a.k != 2 || h->single_tail == 0) return;
   const int E16 = (a.n + 15) / 16;
-  const size_t need = ((size_t)(S.L2 * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
-  if (E16 > kRegVecMaxE || need > 2 * (size_t)a.segStride) return;
+  if (a.Lc != 16 || a.k != 2 || E16 > kRegVecMaxE || h->single_tail == 0) return cudaSuccess;
   const long resident = (long)h->sms * occ * wpb;  // warps the GPU holds at once
   int R = 0;
   if (h->single_tail > 0) {
     R = std::min(pairs, h->single_tail);
-  } else if (4L * pairs <= resident) {
+  } else if (shared ? 3L * pairs <= resident : 4L * pairs <= 3L * resident) {
     R = pairs;  // a small batch: every cell alone, each warp nearly so
   }
-  if (R == 0) return;
+  if (R == 0) return cudaSuccess;
+  const Slots *S = nullptr;
+  const cudaError_t e = view_schedule(v, 16, kOne, nullptr, &S);
+  if (e != cudaSuccess) return e;
+  const size_t need =
+      ((size_t)(S->L * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
+  if (need > 2 * (size_t)a.segStride) return cudaSuccess;
   const int P = pairs - R;
   a.single_from = P;
   a.ngroups = P + std::max(0, a.cells - 2 * P);
-  a.L2 = S.L2;
-  a.sched2 = S.d_words2;
-  a.dst2 = S.d_dst2;
-  a.padfrom2 = S.d_padfrom2;
-  a.dslot2 = S.d_dslot2;
+  a.L2 = S->L;
+  a.sched2 = S->d_words;
+  a.dst2 = S->d_dst;
+  a.pads2 = S->d_pads;
+  a.npads2 = S->npads;
+  a.dslot2 = S->d_dslot;
+  memcpy(a.ends2, S->ends, sizeof a.ends2);
+  return cudaSuccess;
 }
 
 camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
@@ -881,8 +991,9 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
     if (E > kMaxE)
       return fail(CAMP_EUNSUPPORTED, "n=%d needs %d rows per lane at %d lanes per cell (max %d)",
                   v.n, E, Lc, kMaxE);
-    Schedule *S = nullptr;
-    e = view_schedule(v, Lc, &S);
+    Layout *Y = nullptr;
+    const Slots *S = nullptr;
+    e = view_schedule(v, Lc, kAligned, &Y, &S);
     if (e != cudaSuccess) return cuda_fail(e, "schedule upload");
     int wpb = h->wpb > 0 ? h->wpb : 4;
     int segA = 0, segV = 0, segStride = 0;
@@ -895,27 +1006,33 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
       return fail(CAMP_EUNSUPPORTED, "cell does not fit in shared memory (%zu bytes)", smem);
     if (h->wpb == 0 &&
         (e = pick_warps_per_block(v, Lc, S->L, E, 0, h->smem_optin, warp_occupancy,
-                                  &S->auto_wpb[0], &wpb, &smem, &segA, &segV, &segStride)) !=
+                                  &Y->auto_wpb[0], &wpb, &smem, &segA, &segV, &segStride)) !=
             cudaSuccess)
       return cuda_fail(e, "occupancy");
     WarpArgs a = {};
     a.cells = cells; a.n = v.n; a.nnz = v.nnz;
-    a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc; a.L = S->L;
+    a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc;
+    set_slots(a, *S);
     a.segA = segA; a.segV = segV; a.segStride = segStride;
     a.ngroups = (cells + a.k - 1) / a.k;
     a.A = A_vals; a.b = b; a.x = x; a.iters = iters_out; a.resid = resid_out;
-    a.status = status_out; a.sched = S->d_words; a.src = S->d_src;
-    a.dst = S->d_dst; a.padfrom = S->d_padfrom;
-    a.dslot = S->d_dslot; a.tol = tol; a.maxit = maxit;
+    a.status = status_out;
+    a.dslot = S->d_dslot; a.dentry = S->d_dentry; a.tol = tol; a.maxit = maxit;
     a.x0_given = (flags & CAMP_X0_GIVEN) ? 1 : 0;
     a.queue = h->d_queue + 2 * queue_slot;
     a.order = nullptr;
     bool calibrate = false;
     int occ = 0;
-    e = warp_occupancy(E, wpb, smem, &occ);
+    e = warp_occupancy(E, Lc, kTicketsPack, wpb, smem, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy");
     if (occ < 1) occ = 1;
-    set_single_tickets(h, *S, a, wpb, occ);
+    if ((e = set_single_tickets(h, v, a, wpb, occ, queue_slot != 0)) != cudaSuccess)
+      return cuda_fail(e, "schedule upload");
+    if (tickets_of(a) != kTicketsPack) {
+      e = warp_occupancy(E, Lc, tickets_of(a), wpb, smem, &occ);
+      if (e != cudaSuccess) return cuda_fail(e, "occupancy");
+      if (occ < 1) occ = 1;
+    }
     if (queue_slot == 0) {
       const camp_status rs = setup_ordering(h, a, A_vals, smem - sched_smem_bytes(S->L * Lc), st,
                                             &calibrate);
@@ -1033,6 +1150,36 @@ camp_status camp_schedule_build_split(int n, int nnz, const int *row_ptr,
     for (size_t q = 0; q < S.words2.size(); ++q) {
       words[2 * q] = entry[q];
       words[2 * q + 1] = S.words2[q];
+    }
+  }
+  return CAMP_OK;
+}
+
+camp_status camp_schedule_build_aligned(int n, int nnz, const int *row_ptr, const int *col_idx,
+                                        int lanes_per_cell, int split, unsigned *words,
+                                        int capacity_slots, int *slots_per_lane) {
+  int L0 = 0;
+  const camp_status rs =
+      camp_schedule_build(n, nnz, row_ptr, col_idx, lanes_per_cell, nullptr, 0, &L0);
+  if (rs != CAMP_OK) return rs;
+  if (split && lanes_per_cell != 16) return fail(CAMP_EINVAL, "a split layout needs 16 lanes");
+  std::vector<int> rp(row_ptr, row_ptr + n + 1), ci(col_idx, col_idx + nnz), diag(n, -1);
+  for (int i = 0; i < n; ++i)
+    for (int k = rp[i]; k < rp[i + 1]; ++k)
+      if (ci[k] == i) diag[i] = k;
+  Schedule S = build_schedule(n, rp, ci, std::vector<int>(), diag, lanes_per_cell);
+  if (split) split_schedule(S, n, nnz);
+  const int lanes = split ? 32 : lanes_per_cell;
+  std::vector<unsigned> word;
+  std::vector<int> src;
+  const int L = sched::align(n, row_chains(S, rp), lanes, split ? S.L2 : S.L, word, src);
+  *slots_per_lane = L;
+  if (words && L) {
+    if ((long)L * lanes > (long)capacity_slots)
+      return fail(CAMP_EINVAL, "capacity %d < %d slots", capacity_slots, L * lanes);
+    for (size_t q = 0; q < word.size(); ++q) {
+      words[2 * q] = (unsigned)src[q];
+      words[2 * q + 1] = word[q];
     }
   }
   return CAMP_OK;
@@ -1461,20 +1608,22 @@ namespace {
 
 // Per-lane term lists of the handle's mechanism for Lc lanes per cell, padded
 // to the longest lane and laid out [term][lane]: the Jacobian terms of the
-// lane's slots (tmeta = (species + 1) | slot row << 11) and the rate terms of
+// lane's slots (tmeta = (species + 1) | place << 11) and the rate terms of
 // the lane's rows (rmeta = (a + 1) | (b + 1) << 11 | e << 22, row sl + e Lc).
-cudaError_t mech_terms(Mechanism &mech, int Lc, const Schedule &S, MechTerms **out) {
+cudaError_t mech_terms(Mechanism &mech, int Lc, const Slots &S, MechTerms **out) {
   auto it = mech.by_lanes.find(Lc);
   if (it != mech.by_lanes.end()) {
     *out = &it->second;
     return cudaSuccess;
   }
   auto pad = [Lc](std::vector<std::vector<std::pair<double, int>>> &lane,
-                  std::vector<double> &val, std::vector<int> &meta) {
+                  std::vector<double> &val, std::vector<int> &meta, auto idle) {
     size_t M = 1;
     for (auto &l : lane) M = std::max(M, l.size());
     val.assign(M * Lc, 0.0);
     meta.assign(M * Lc, 0);
+    for (size_t p = 0; p < M; ++p)
+      for (int q = 0; q < Lc; ++q) meta[p * Lc + q] = idle(q);
     for (int q = 0; q < Lc; ++q)
       for (size_t p = 0; p < lane[q].size(); ++p) {
         val[p * Lc + q] = lane[q][p].first;
@@ -1485,7 +1634,8 @@ cudaError_t mech_terms(Mechanism &mech, int Lc, const Schedule &S, MechTerms **o
   std::vector<std::vector<std::pair<double, int>>> lane(Lc), rlane(Lc);
   for (size_t q = 0; q < mech.entry.size(); ++q) {
     const int t = S.dst[mech.entry[q]];
-    lane[t % Lc].push_back({mech.val[q], (mech.spec[q] + 1) | ((t / Lc) << 11)});
+    lane[t % Lc].push_back(
+        {mech.val[q], (mech.spec[q] + 1) | (pair_pos(t / Lc, t % Lc, S.L, Lc) << 11)});
   }
   for (size_t q = 0; q < mech.rrow.size(); ++q) {
     const int row = mech.rrow[q];
@@ -1495,8 +1645,9 @@ cudaError_t mech_terms(Mechanism &mech, int Lc, const Schedule &S, MechTerms **o
   std::vector<double> tval, rval;
   std::vector<int> tmeta, rmeta;
   MechTerms T;
-  T.count = pad(lane, tval, tmeta);
-  T.rcount = pad(rlane, rval, rmeta);
+  // a padding term adds zero to a place (a row) of its own lane
+  T.count = pad(lane, tval, tmeta, [&](int q) { return pair_pos(0, q, S.L, Lc) << 11; });
+  T.rcount = pad(rlane, rval, rmeta, [](int) { return 0; });
   cudaError_t e;
   if ((e = upload(&T.d_tval, tval)) != cudaSuccess ||
       (e = upload(&T.d_tmeta, tmeta)) != cudaSuccess ||
@@ -1523,8 +1674,10 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
   const int E = Lc ? (v.n + Lc - 1) / Lc : 0;
   if (Lc == 0 || E > 8)
     return fail(CAMP_EUNSUPPORTED, "fused assembly supports at most 8 rows per lane (n=%d)", v.n);
-  Schedule *S = nullptr;
-  if ((e = view_schedule(v, Lc, &S)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+  Layout *Y = nullptr;
+  const Slots *S = nullptr;
+  if ((e = view_schedule(v, Lc, kAligned, &Y, &S)) != cudaSuccess)
+    return cuda_fail(e, "schedule upload");
   if (S->L > 2047) return fail(CAMP_EUNSUPPORTED, "more than 2047 slots per lane");
   MechTerms *T = nullptr;
   if ((e = mech_terms(h->mech, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
@@ -1536,16 +1689,16 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
   if (smem > h->smem_optin) return fail(CAMP_EUNSUPPORTED, "cell does not fit in shared memory");
   if (h->wpb == 0 &&
       (e = pick_warps_per_block(v, Lc, S->L, E, extra_vectors, h->smem_optin, occ_fn,
-                                &S->auto_wpb[extra_vectors ? 2 : 1], &wpb, &smem, &segA, &segV,
+                                &Y->auto_wpb[extra_vectors ? 2 : 1], &wpb, &smem, &segA, &segV,
                                 &segStride)) != cudaSuccess)
     return cuda_fail(e, "occupancy");
   WarpArgs a = {};
   a.cells = cells; a.n = v.n; a.nnz = v.nnz;
-  a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc; a.L = S->L;
+  a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc;
+  set_slots(a, *S);
   a.segA = segA; a.segV = segV; a.segStride = segStride;
   a.ngroups = (cells + a.k - 1) / a.k;
-  a.sched = S->d_words; a.src = S->d_src;
-  a.dst = S->d_dst; a.padfrom = S->d_padfrom; a.dslot = S->d_dslot;
+  a.dslot = S->d_dslot;
   a.x0_given = 0;
   a.queue = h->d_queue;
   a.tval = T->d_tval; a.tmeta = T->d_tmeta; a.tcount = T->count;
@@ -1580,7 +1733,7 @@ camp_status camp_solver_assemble_solve(camp_solver_t h, int cells,
   a.conc = conc; a.gamma = gamma;
   int occ = 0;
   cudaError_t e;
-  if ((e = assemble_occupancy(E, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
+  if ((e = assemble_occupancy(E, a.Lc, kTicketsPack, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min((a.ngroups + wpb - 1) / wpb, h->sms * occ));
   rc = setup_gamma_ordering(h, a, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
@@ -1627,7 +1780,7 @@ camp_status camp_solver_newton_solve(camp_solver_t h, int cells,
   a.newton_iters = newton_iters_out; a.upd = upd_out;
   int occ = 0;
   cudaError_t e;
-  if ((e = newton_occupancy(E, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
+  if ((e = newton_occupancy(E, a.Lc, kTicketsPack, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min((a.ngroups + wpb - 1) / wpb, h->sms * occ));
   rc = setup_gamma_ordering(h, a, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
@@ -1664,8 +1817,9 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
   if (Lc == 0) return fail(CAMP_EUNSUPPORTED, "no warp arrangement fits n=%d", v.n);
   const int E = (v.n + Lc - 1) / Lc;
   if (E > kMaxE) return fail(CAMP_EUNSUPPORTED, "n=%d too large for %d lanes per cell", v.n, Lc);
-  Schedule *S = nullptr;
-  if ((e = view_schedule(v, Lc, &S)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+  const Slots *S = nullptr;
+  if ((e = view_schedule(v, Lc, kPlain, nullptr, &S)) != cudaSuccess)
+    return cuda_fail(e, "schedule upload");
   // FP64 A in shared memory unless that costs resident warps (then the
   // outer residual product reads it through L1)
   const int wpb0 = h->wpb > 0 ? h->wpb : 4;
@@ -1689,11 +1843,12 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
   smem = mixed_smem(v, Lc, S->L, wpb, &segA, &segV, a64);
   MixedArgs a = {};
   a.cells = cells; a.n = v.n; a.nnz = v.nnz;
-  a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc; a.L = S->L;
+  a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc;
+  set_slots(a, *S);
   a.segA = segA; a.segV = segV; a.ngroups = (cells + a.k - 1) / a.k;
   a.A = A_vals; a.b = b; a.x = x; a.iters = iters_out; a.sweeps = sweeps_out;
-  a.resid = resid_out; a.status = status_out; a.sched = S->d_words; a.src = S->d_src;
-  a.dst = S->d_dst; a.padfrom = S->d_padfrom; a.dslot = S->d_dslot;
+  a.resid = resid_out; a.status = status_out;
+  a.dst32 = S->d_dst32; a.pads32 = S->d_pads32; a.dslot32 = S->d_dslot32;
   a.tol = tol; a.max_sweeps = max_sweeps; a.tol_in = (float)tol_inner;
   a.maxit_in = maxit_inner;
   a.a64_smem = a64 ? 1 : 0;
@@ -1874,19 +2029,20 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
     View &v = h->fwd;
     int Lc = 1;
     while ((v.n + Lc - 1) / Lc > E) Lc *= 2;
-    Schedule *S = nullptr;
-    if ((e = view_schedule(v, Lc, &S)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+    const Slots *S = nullptr;
+    if ((e = view_schedule(v, Lc, kAligned, nullptr, &S)) != cudaSuccess)
+      return cuda_fail(e, "schedule upload");
     WarpArgs &a = args.m[q];
     a.cells = cells[m]; a.n = v.n; a.nnz = v.nnz;
-    a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc; a.L = S->L;
+    a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc;
+    set_slots(a, *S);
     a.segA = asmem ? ((S->L * Lc + 1) & ~1) : 0;
     a.segV = ((E * Lc + 1) + 1) & ~1;
     a.segStride = bank_spread_stride(a.segA + warp_vectors(E) * a.segV, a.k);
     a.ngroups = (cells[m] + a.k - 1) / a.k;
     a.A = A_vals[m]; a.b = bvec[m]; a.x = x[m]; a.iters = iters_out[m];
     a.resid = resid_out[m]; a.status = status_out ? status_out[m] : nullptr;
-    a.sched = S->d_words; a.src = S->d_src; a.dslot = S->d_dslot;
-    a.dst = S->d_dst; a.padfrom = S->d_padfrom;
+    a.dslot = S->d_dslot; a.dentry = S->d_dentry;
     a.tol = tol; a.maxit = maxit; a.x0_given = 0; a.queue = nullptr;
     args.item_begin[q] = items;
     items += a.ngroups;
@@ -2051,9 +2207,11 @@ namespace {
 
 std::mutex g_noalloc_mu;                              // guards the host buffers below
 void *g_noalloc_dev[kNoAllocMaxDevices];              // device address of the scratch
-SchedWord g_noalloc_words[kNoAllocScratchBytes / sizeof(SchedWord)];
+unsigned g_noalloc_words[kNoAllocScratchBytes / sizeof(unsigned)];      // host form
+SchedWord g_noalloc_packed[kNoAllocScratchBytes / sizeof(SchedWord)];  // device form
 int g_noalloc_dst[kNoAllocScratchBytes / sizeof(int)];
 int g_noalloc_padfrom[32];
+unsigned g_noalloc_ends[kEndWords];
 int g_noalloc_entry[kNoAllocScratchBytes / sizeof(SchedWord)];
 int g_noalloc_order[1024], g_noalloc_diag[1024], g_noalloc_dslot[1024];
 int g_noalloc_bin_rows[32][1024], g_noalloc_bin_count[32];
@@ -2073,8 +2231,16 @@ int noalloc_schedule(int n, const int *rp, const int *ci, int Lc, size_t cap_slo
   const int L = sched::build(n, rp, ci, g_noalloc_diag, Lc, cap, w, g_noalloc_words,
                              g_noalloc_entry, g_noalloc_dslot, g_noalloc_padfrom);
   if (L < 0) return -1;
-  for (long t = 0; t < (long)L * Lc; ++t)
-    if (g_noalloc_entry[t] >= 0) g_noalloc_dst[g_noalloc_entry[t]] = (int)t;
+  // device form: places instead of slot numbers
+  for (int j = 0; j < L; ++j)
+    for (int q = 0; q < Lc; ++q) {
+      const int k = g_noalloc_entry[(size_t)j * Lc + q];
+      if (k >= 0) g_noalloc_dst[k] = pair_pos(j, q, L, Lc);
+    }
+  for (int r = 0; r < n; ++r)
+    g_noalloc_dslot[r] = pair_pos(g_noalloc_dslot[r] / Lc, g_noalloc_dslot[r] % Lc, L, Lc);
+  sched::pack_words(L, Lc, g_noalloc_words, g_noalloc_packed);
+  sched::end_mask(L, Lc, g_noalloc_words, g_noalloc_ends);
   return L;
 }
 
@@ -2169,7 +2335,9 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
   a.A = A_vals; a.b = b; a.x = x; a.iters = iters_out; a.resid = resid_out;
   a.status = status_out;
   a.dslot = (const int *)scratch;
-  a.padfrom = (const int *)(scratch + diag_bytes);
+  a.pads = (const int *)(scratch + diag_bytes);
+  a.npads = -1;  // per lane: the first padding slot
+  memcpy(a.ends, g_noalloc_ends, sizeof a.ends);
   a.dst = (const int *)(scratch + diag_bytes + pad_bytes);
   a.sched = (const SchedWord *)(scratch + head_bytes);
   a.src = nullptr;  // only the global-memory A path reads it
@@ -2180,7 +2348,7 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
   while (smem > (size_t)optin && wpb > 1) smem = sch + (size_t)(--wpb) * a.k * a.segStride * 8;
   if (smem > (size_t)optin) return fail(CAMP_EUNSUPPORTED, "cell does not fit in shared memory");
   int occ = 0;
-  if ((e = warp_occupancy(E, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
+  if ((e = warp_occupancy(E, Lc, kTicketsPack, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min((a.ngroups + wpb - 1) / wpb, sms * occ));
   // stage the schedule pieces (pageable source: each call returns once its
@@ -2191,7 +2359,7 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
                            cudaMemcpyHostToDevice, st)) != cudaSuccess ||
       (e = cudaMemcpyAsync(scratch + diag_bytes + pad_bytes, g_noalloc_dst,
                            (size_t)nnz * sizeof(int), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(scratch + head_bytes, g_noalloc_words,
+      (e = cudaMemcpyAsync(scratch + head_bytes, g_noalloc_packed,
                            (size_t)L * Lc * sizeof(SchedWord), cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(e, "staging into the static scratch");
   if ((e = launch_warp(E, a, wpb, grid, smem, st)) != cudaSuccess)

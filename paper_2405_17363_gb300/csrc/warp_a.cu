@@ -2,8 +2,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_WARP_DEFINE(1)
-CAMP_WARP_DEFINE(2)
-CAMP_WARP_DEFINE(3)
-CAMP_WARP_DEFINE(4)
+CAMP_KERNEL_DEFINE(warp, 1)
+CAMP_KERNEL_DEFINE(warp, 2)
+CAMP_KERNEL_DEFINE(warp, 3)
+CAMP_KERNEL_DEFINE(warp, 4)
 }  // namespace camp

@@ -2,8 +2,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_WARP_DEFINE(5)
-CAMP_WARP_DEFINE(6)
-CAMP_WARP_DEFINE(7)
-CAMP_WARP_DEFINE(8)
+CAMP_KERNEL_DEFINE(warp, 5)
+CAMP_KERNEL_DEFINE(warp, 6)
+CAMP_KERNEL_DEFINE(warp, 7)
+CAMP_KERNEL_DEFINE(warp, 8)
 }  // namespace camp

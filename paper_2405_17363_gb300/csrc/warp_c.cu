@@ -2,8 +2,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_WARP_DEFINE(9)
-CAMP_WARP_DEFINE(10)
-CAMP_WARP_DEFINE(11)
-CAMP_WARP_DEFINE(12)
+CAMP_KERNEL_DEFINE(warp, 9)
+CAMP_KERNEL_DEFINE(warp, 10)
+CAMP_KERNEL_DEFINE(warp, 11)
+CAMP_KERNEL_DEFINE(warp, 12)
 }  // namespace camp

@@ -7,7 +7,6 @@
 namespace camp {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kSpmvUnroll = 4;  // SpMV pipeline block (slots per lane)
 
 // Difficulty class of a cell from the high word of its estimate
 // max_i |A_ii - 1| (a non-negative double, so its high words order as
@@ -70,116 +69,161 @@ __device__ __forceinline__ void seg_sum2(double &a, double &b, int Lc) {
   b = up ? keep : other;
 }
 
-// Three sums (a fourth slot is zero) with two transposing levels: 2 + 1 +
-// (log2(Lc) - 2) FP64 additions for Lc >= 4.
-__device__ __forceinline__ void seg_sum3(double &a, double &b, double &c, int Lc) {
-  if (Lc < 4) {
-    double v[3] = {a, b, c};
-    seg_sum<3>(v, Lc);
-    a = v[0]; b = v[1]; c = v[2];
-    return;
-  }
-  const int h1 = Lc >> 1, h2 = Lc >> 2;
-  const bool u1 = (threadIdx.x & h1) != 0;
-  const bool u2 = (threadIdx.x & h2) != 0;
-  // level 1: lower half keeps (a, b), upper half keeps (c, 0)
-  double k0 = u1 ? c : a, k1 = u1 ? 0.0 : b;
-  const double s0 = u1 ? a : c, s1 = u1 ? b : 0.0;
-  k0 += __shfl_xor_sync(kFull, s0, h1);
-  k1 += __shfl_xor_sync(kFull, s1, h1);
-  // level 2: lower quarter keeps k0, upper keeps k1
-  double k = u2 ? k1 : k0;
-  const double s = u2 ? k0 : k1;
-  k += __shfl_xor_sync(kFull, s, h2);
-  for (int off = h2 >> 1; off > 0; off >>= 1) k += __shfl_xor_sync(kFull, k, off);
-  // lane classes (u1, u2): (0,0) a, (0,1) b, (1,0) c, (1,1) zero
-  const double x2 = __shfl_xor_sync(kFull, k, h2);
-  const double x1 = __shfl_xor_sync(kFull, k, h1);
-  const double x3 = __shfl_xor_sync(kFull, k, h1 | h2);
-  // the lane whose class is (p, q) holds: own k, x2 = (p, !q), x1 = (!p, q), x3 = (!p, !q)
-  const double va = (!u1 && !u2) ? k : (!u1 && u2) ? x2 : (u1 && !u2) ? x1 : x3;
-  const double vb = (!u1 && u2) ? k : (!u1 && !u2) ? x2 : (u1 && u2) ? x1 : x3;
-  const double vc = (u1 && !u2) ? k : (u1 && u2) ? x2 : (!u1 && !u2) ? x1 : x3;
-  a = va; b = vb; c = vc;
-}
-
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
 
-// *p = v when flag != 0, as one predicated shared-memory store (no branch)
-__device__ __forceinline__ void store_if(unsigned flag, double *p, double v) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+// Shared-memory accesses by 32-bit address (byte offset in the CTA's window).
+__device__ __forceinline__ unsigned smem_addr(const void *p) {
+  return (unsigned)__cvta_generic_to_shared(p);
+}
+__device__ __forceinline__ void lds(double &v, unsigned a) {
+  asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a));
+}
+__device__ __forceinline__ void lds(float &v, unsigned a) {
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
+}
+// *a = v when flag != 0, as one predicated store (no branch)
+__device__ __forceinline__ void sts_if(unsigned flag, unsigned a, double v) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.f64 [%1], %2;\n\t}"
                :: "r"(flag), "r"(a), "d"(v) : "memory");
 }
-__device__ __forceinline__ void store_if(unsigned flag, float *p, float v) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+__device__ __forceinline__ void sts_if(unsigned flag, unsigned a, float v) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.f32 [%1], %2;\n\t}"
                :: "r"(flag), "r"(a), "f"(v) : "memory");
 }
 
-// os[row] = sum over this lane's slots of A_slot * gs[col] (os: shared
-// memory).  sch and loadA(j) give this lane's word and A value of slot j.
-// Software pipeline over blocks of P slots: the block's A values and gathers
-// (its words were read one block earlier) and the next block's words are
-// issued before the block's chain of multiply-adds, so the shared-memory
-// latency runs under the FP64 chain; a row end is a predicated store and a
-// select, without a branch.  Slots past L read word 0 and A = 0 (no row end
-// follows them).
-template <class T, class LoadA>
-__device__ __forceinline__ void spmv_slots(const SchedWord *__restrict__ sch, int L, int Lc,
-                                           LoadA loadA, const T *__restrict__ gs,
-                                           T *__restrict__ os) {
-  constexpr int P = kSpmvUnroll;
-  SchedWord w[P];
-#pragma unroll
-  for (int u = 0; u < P; ++u) w[u] = u < L ? sch[u * Lc] : 0u;
+// The gathered vector's address of a slot (a word holds 4 * column above 4 *
+// row and the lane's end flag).
+template <class T>
+__device__ __forceinline__ unsigned slot_col_addr(unsigned w, unsigned gs) {
+  return gs + (w >> (sizeof(T) == 8 ? 15 : 16));
+}
+// A slot in which some lane ends a row: those lanes store their sum and
+// start from zero (a predicated store and a select).
+template <class T>
+__device__ __forceinline__ void slot_end(unsigned w, T &acc, unsigned os) {
+  sts_if(w & kSlotEnd, os + (w & kSlotRowMask) * (sizeof(T) == 8 ? 2u : 1u), acc);
+  acc = (w & kSlotEnd) ? T(0) : acc;
+}
+
+// os[row] = sum over this lane's slots of A_slot * gs[col] (gs, os: shared
+// addresses; sch: the schedule's words; ends: the launch's row-end mask, a
+// kernel parameter, so the tests on it are uniform branches).  lo(b, ..) and
+// hi(b, ..) give the A values of the lane's slots 4b, 4b+1 and 4b+2, 4b+3;
+// last(j, av), those of the slots j .. L-1 past the last whole block.
+// FP64: the chain of dependent multiply-adds (64 cycles each for one warp,
+// which is also the sub-partition's issue interval) bounds both a lone warp
+// and a full SM, so everything else runs under it: the gathers and A values
+// of a half block are issued two multiply-adds ahead, the words a block
+// ahead, and only the slots of the end mask (8 or 9 of 36 at 80 rows on 16
+// lanes) put a select on the chain.  Measured at 80 rows, 564 entries, 16
+// lanes: 76 cycles per slot for a lone warp against 100 with a conditional
+// store and select in every slot, 65 per slot and warp with four warps per
+// sub-partition either way.
+template <class T, class Lo, class Hi, class Last>
+__device__ __forceinline__ void spmv_slots(const SchedWord *__restrict__ sch,
+                                           const unsigned *__restrict__ ends, int L, int Lc, int sl,
+                                           Lo lo, Hi hi, Last last, unsigned gs, unsigned os) {
+  static_assert(kSlotBlock == 4, "word blocks are 16 bytes");
+  const uint4 *s4 = reinterpret_cast<const uint4 *>(sch) + sl;
   T acc = T(0);
-  for (int j0 = 0; j0 < L; j0 += P) {
-    T av[P], xv[P];
-    SchedWord wn[P];
-#pragma unroll
-    for (int u = 0; u < P; ++u) {
-      av[u] = j0 + u < L ? loadA(j0 + u) : T(0);
-      xv[u] = gs[w[u] & 0x7ffu];
+  const int nb = L >> 2;
+  unsigned mk = 0;
+  if (nb > 0) {
+    uint4 w = *s4;
+    T x0, x1, x2, x3, a0, a1, a2, a3;
+    lds(x0, slot_col_addr<T>(w.x, gs));
+    lds(x1, slot_col_addr<T>(w.y, gs));
+    lo(0, a0, a1);
+#pragma unroll 1
+    for (int b = 0;;) {
+      if ((b & 7) == 0) mk = b < 8 * kEndWords ? ends[b >> 3] : ~0u;
+      lds(x2, slot_col_addr<T>(w.z, gs));
+      lds(x3, slot_col_addr<T>(w.w, gs));
+      hi(b, a2, a3);
+      uint4 wn = w;
+      const bool more = ++b < nb;
+      if (more) wn = s4[b * Lc];
+      acc = fma_t(a0, x0, acc);
+      if (mk & 1u) slot_end(w.x, acc, os);
+      acc = fma_t(a1, x1, acc);
+      if (mk & 2u) slot_end(w.y, acc, os);
+      if (more) {
+        lds(x0, slot_col_addr<T>(wn.x, gs));
+        lds(x1, slot_col_addr<T>(wn.y, gs));
+        lo(b, a0, a1);
+      }
+      acc = fma_t(a2, x2, acc);
+      if (mk & 4u) slot_end(w.z, acc, os);
+      acc = fma_t(a3, x3, acc);
+      if (mk & 8u) slot_end(w.w, acc, os);
+      mk >>= 4;
+      if (!more) break;
+      w = wn;
     }
+  }
+  if (L & 3) {
+    if ((nb & 7) == 0) mk = nb < 8 * kEndWords ? ends[nb >> 3] : ~0u;
+    SchedWord w[3];
+    T av[3], xv[3];
 #pragma unroll
-    for (int u = 0; u < P; ++u) {
-      const int j = j0 + P + u;
-      wn[u] = j < L ? sch[j * Lc] : 0u;
-    }
+    for (int u = 0; u < 3; ++u) w[u] = (L & 3) > u ? sch[(4 * nb + u) * Lc + sl] : 0u;
 #pragma unroll
-    for (int u = 0; u < P; ++u) {
-      acc = fma_t(av[u], xv[u], acc);
-      store_if(w[u] & kSlotEnd, os + ((w[u] >> 11) & 0x7ffu), acc);
-      acc = (w[u] & kSlotEnd) ? T(0) : acc;
-    }
+    for (int u = 0; u < 3; ++u) lds(xv[u], slot_col_addr<T>(w[u], gs));
+    last(4 * nb, av);
 #pragma unroll
-    for (int u = 0; u < P; ++u) w[u] = wn[u];
+    for (int u = 0; u < 3; ++u)
+      if ((L & 3) > u) {
+        acc = fma_t(av[u], xv[u], acc);
+        if (mk & (1u << u)) slot_end(w[u], acc, os);
+      }
   }
 }
 
-// o[row] = sum over this lane's slots of A_slot * g[col].  sch and As point at
-// this lane's column of the schedule and of the slot-ordered A (stride Lc).
+// o[row] = sum over this lane's slots of A_slot * g[col], A in slot order in
+// shared memory (As: the cell's block, pair_pos places).
 __device__ __forceinline__ void seg_spmv(const SchedWord *__restrict__ sch,
-                                         int L, int Lc,
-                                         const double *__restrict__ As,
-                                         const double *__restrict__ gs,
-                                         double *__restrict__ os) {
-  spmv_slots<double>(sch, L, Lc, [&](int j) { return As[j * Lc]; }, gs, os);
+                                         const unsigned *__restrict__ ends, int L, int Lc, int sl,
+                                         const double *__restrict__ As, unsigned gs, unsigned os) {
+  const double2 *A2 = reinterpret_cast<const double2 *>(As) + sl;
+  auto pair = [&](int p, double &a, double &b) {
+    const double2 v = A2[p * Lc];
+    a = v.x;
+    b = v.y;
+  };
+  spmv_slots<double>(
+      sch, ends, L, Lc, sl, [&](int b, double &u, double &v) { pair(2 * b, u, v); },
+      [&](int b, double &u, double &v) { pair(2 * b + 1, u, v); },
+      [&](int j, double *av) {
+        if (L - j > 1) pair(j >> 1, av[0], av[1]);
+        else av[0] = As[j * Lc + sl];
+        if (L - j > 2) av[2] = As[(j + 2) * Lc + sl];
+      },
+      gs, os);
 }
 
-// Same with A read from global memory through the slot's source entry.
+// Same with A read from global memory through the slots' source entries.
 __device__ __forceinline__ void seg_spmv_gather(const SchedWord *__restrict__ sch,
-                                                const int *__restrict__ src,
-                                                int L, int Lc,
-                                                const double *__restrict__ Ag,
-                                                const double *__restrict__ gs,
-                                                double *__restrict__ os) {
-  spmv_slots<double>(sch, L, Lc, [&](int j) {
-    const int k = __ldg(src + j * Lc);
-    return k >= 0 ? __ldg(Ag + k) : 0.0;
-  }, gs, os);
+                                                const unsigned *__restrict__ ends,
+                                                const int *__restrict__ src, int L, int Lc, int sl,
+                                                const double *__restrict__ Ag, unsigned gs,
+                                                unsigned os) {
+  const int2 *s2 = reinterpret_cast<const int2 *>(src) + 2 * sl;
+  auto value = [&](int k) { return k >= 0 ? __ldg(Ag + k) : 0.0; };
+  auto pair = [&](int p, double &a, double &b) {
+    const int2 k = __ldg(s2 + (p >> 1) * 2 * Lc + (p & 1));
+    a = value(k.x);
+    b = value(k.y);
+  };
+  spmv_slots<double>(
+      sch, ends, L, Lc, sl, [&](int b, double &u, double &v) { pair(2 * b, u, v); },
+      [&](int b, double &u, double &v) { pair(2 * b + 1, u, v); },
+      [&](int j, double *av) {
+#pragma unroll
+        for (int u = 0; u < 3; ++u)
+          if (L - j > u) av[u] = value(__ldg(src + (j + u) * Lc + sl));
+      },
+      gs, os);
 }
 
 // Coalesced, vectorised read of one cell's A row (CSR order), handed to
@@ -221,11 +265,14 @@ __device__ __forceinline__ void stage_scatter(const double *__restrict__ Ac,
   }
 }
 
-// Zero this lane's padding slots of a slot-ordered A (never scatter targets).
+// Zero a slot-ordered A's padding slots (never scatter targets): the places
+// pads[0 .. npads), or with npads < 0 every lane's slots from pads[lane] on.
 template <class T>
-__device__ __forceinline__ void zero_padding(T *__restrict__ Abase, const int *__restrict__ padfrom,
-                                             int L, int Lc, int sl) {
-  for (int t = __ldg(padfrom + sl) * Lc + sl; t < L * Lc; t += Lc) Abase[t] = T(0);
+__device__ __forceinline__ void zero_padding(T *__restrict__ Abase, const int *__restrict__ pads,
+                                             int npads, int L, int sl, int Lc) {
+  for (int i = sl; i < npads; i += Lc) Abase[__ldg(pads + i)] = T(0);
+  if (npads < 0)
+    for (int j = __ldg(pads + sl); j < L; ++j) Abase[pair_pos(j, sl, L, Lc)] = T(0);
 }
 
 // float variant of the segment sum
@@ -237,13 +284,48 @@ __device__ __forceinline__ void seg_sumf(float (&v)[NV], int Lc) {
   }
 }
 
-// FP32 variant (slot-ordered A32).
-__device__ __forceinline__ void seg_spmvf(const SchedWord *__restrict__ sch,
-                                          int L, int Lc,
-                                          const float *__restrict__ As,
-                                          const float *__restrict__ gs,
-                                          float *__restrict__ os) {
-  spmv_slots<float>(sch, L, Lc, [&](int j) { return As[j * Lc]; }, gs, os);
+// The FP32 product (A32 in slot order, word_pos places), with a row end in
+// every slot (a predicated store and a select, no branch): an FP32 chain is
+// short, so issue slots bound it, and the branches of spmv_slots cost more
+// than they save (150 species x 100,000 cells: 1,983 us against 2,195).
+__device__ __forceinline__ void seg_spmvf(const SchedWord *__restrict__ sch, int L, int Lc, int sl,
+                                          const float *__restrict__ As, unsigned gs, unsigned os) {
+  const uint4 *s4 = reinterpret_cast<const uint4 *>(sch) + sl;
+  const float4 *A4 = reinterpret_cast<const float4 *>(As) + sl;
+  float acc = 0.0f;
+  const int nb = L >> 2;
+  auto step = [&](unsigned w, float av, float xv) {
+    acc = fma_t(av, xv, acc);
+    slot_end(w, acc, os);
+  };
+  if (nb > 0) {
+    uint4 w = *s4;
+#pragma unroll 1
+    for (int b = 0;;) {
+      float x0, x1, x2, x3;
+      lds(x0, slot_col_addr<float>(w.x, gs));
+      lds(x1, slot_col_addr<float>(w.y, gs));
+      lds(x2, slot_col_addr<float>(w.z, gs));
+      lds(x3, slot_col_addr<float>(w.w, gs));
+      const float4 av = A4[b * Lc];
+      uint4 wn = w;
+      if (++b < nb) wn = s4[b * Lc];
+      step(w.x, av.x, x0);
+      step(w.y, av.y, x1);
+      step(w.z, av.z, x2);
+      step(w.w, av.w, x3);
+      if (b == nb) break;
+      w = wn;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if ((L & 3) > u) {
+      const unsigned w = sch[(4 * nb + u) * Lc + sl];
+      float x;
+      lds(x, slot_col_addr<float>(w, gs));
+      step(w, As[(4 * nb + u) * Lc + sl], x);
+    }
 }
 
 // FP64 -> FP32 conversion, round to nearest even, entirely on the integer

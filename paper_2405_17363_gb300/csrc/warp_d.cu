@@ -2,8 +2,8 @@
 #include "warp_kernel.cuh"
 #include "warp_launch.cuh"
 namespace camp {
-CAMP_WARP_DEFINE(13)
-CAMP_WARP_DEFINE(14)
-CAMP_WARP_DEFINE(15)
-CAMP_WARP_DEFINE(16)
+CAMP_KERNEL_DEFINE(warp, 13)
+CAMP_KERNEL_DEFINE(warp, 14)
+CAMP_KERNEL_DEFINE(warp, 15)
+CAMP_KERNEL_DEFINE(warp, 16)
 }  // namespace camp

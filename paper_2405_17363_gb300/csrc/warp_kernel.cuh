@@ -48,20 +48,14 @@ __device__ __forceinline__ void ssum2(double &a, double &b, int Lc) {
     seg_sum2(a, b, Lc);
   }
 }
-template <int LC>
-__device__ __forceinline__ void ssum3(double &a, double &b, double &c, int Lc) {
-  if (CAMP_EXACT_SUMS) {
-    a = seg_sum_x<LC>(a, Lc);
-    b = seg_sum_x<LC>(b, Lc);
-    c = seg_sum_x<LC>(c, Lc);
-  } else {
-    seg_sum3(a, b, c, Lc);
-  }
-}
-
-#ifndef CAMP_WARP_MINB
-#define CAMP_WARP_MINB 2  // with 256 threads per CTA at most: <= 128 registers
-#endif
+// At most 168 registers: 12 warps per SM (the CTAs themselves have at most 8).
+// Two warps keep a sub-partition's FP64 unit 97 % busy (11,160 cycles per
+// iteration and warp against 10,845 with four), so registers are worth more
+// than a fourth warp: with 128 the kernels spill, and the fewer groups in
+// flight when the queue runs dry, the sooner the launch ends.  80 species x
+// 10,000 cells: 187 us against 197 with 16 warps and 128 registers; 150
+// species x 50,000: 1,698 against 1,756.
+#define CAMP_WARP_BOUNDS __launch_bounds__(384, 1)
 
 // Where a group's matrix values come from (template parameter SRC of
 // solve_group): staged from A into shared memory in slot order, read from A
@@ -188,8 +182,8 @@ __device__ __forceinline__ void newton_loop(const WarpArgs &a, bool has, bool &l
 }
 
 // Solve the k = 32/Lc cells of group g (cells g*k .. g*k+k-1) of one
-// mechanism with this warp.  wbase: the warp's shared-memory region; sch: this
-// lane's column of the SpMV schedule (shared or global memory).
+// mechanism with this warp.  wbase: the warp's shared-memory region; sch: the
+// SpMV schedule's words (shared or global memory).
 template <int E, int SRC, int LC = 0>
 __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
                                             double *wbase,
@@ -222,14 +216,12 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
                     : pos;
 #define SPMV(out)                                                    \
   do {                                                               \
-    if (ASMEM) seg_spmv(sch, a.L, Lc, Asl, gs, out);                 \
-    else seg_spmv_gather(sch, srcl, a.L, Lc, Ac, gs, out);           \
+    if (ASMEM) seg_spmv(sch, a.ends, a.L, Lc, sl, Abase, gsa, smem_addr(out)); \
+    else seg_spmv_gather(sch, a.ends, a.src, a.L, Lc, sl, Ac, gsa, smem_addr(out)); \
   } while (0)
   const double *Ac = a.A + (size_t)(has ? c : 0) * nnz;
-  const int *srcl = a.src + sl;
-  const int LL = a.L * Lc;
   constexpr bool ASMEM = SRC != kSrcGlobal;
-  const double *Asl = Abase + sl;  // this lane's slots (stride Lc)
+  const unsigned gsa = smem_addr(gs);
   double xv[E];
   int st = -1, it = 0;
   double resid = 0.0;
@@ -246,7 +238,7 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   // one team); the transposed view's permutation is folded into src
   if (SRC == kSrcAssembled || SRC == kSrcNewton) {
     // J accumulates in place in the lane's own slots, then A = I - gamma J
-    for (int t = sl; t < LL; t += Lc) Abase[t] = 0.0;
+    for (int j = 0; j < a.L; ++j) Abase[pair_pos(j, sl, a.L, Lc)] = 0.0;
     // the cell's concentrations go to the (not yet used) t-product buffer
     // (the Newton launch has put the current iterate there)
     if (SRC == kSrcAssembled && live)
@@ -258,19 +250,21 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
     for (int p = 0; p < a.tcount; ++p) {
       const int meta = __ldg(tm + p * Lc);
       const int sp = (meta & 0x7ff) - 1;
-      double *dst = Abase + ((meta >> 11) & 0x7ff) * Lc + sl;
+      double *dst = Abase + (meta >> 11);
       *dst = fma(__ldg(tv + p * Lc), sp >= 0 ? o2[sp] : 1.0, *dst);
     }
-    for (int t = sl; t < LL; t += Lc) {
-      const SchedWord w = sch[t - sl];  // this lane's word for slot t
-      const bool dg = __ldg(a.src + t) >= 0 && (w & 0x7ffu) == ((w >> 11) & 0x7ffu);
-      Abase[t] = fma(-gam, Abase[t], dg ? 1.0 : 0.0);
+    for (int j = 0; j < a.L; ++j) {
+      const SchedWord w = sch[word_pos(j, sl, a.L, Lc)];  // this lane's word for slot j
+      const bool dg = __ldg(a.src + word_pos(j, sl, a.L, Lc)) >= 0 &&
+                      (w & kSlotRowMask) == (w >> 16);
+      double *t = Abase + pair_pos(j, sl, a.L, Lc);
+      *t = fma(-gam, *t, dg ? 1.0 : 0.0);
     }
   } else if (ASMEM) {
     // coalesced read of the cell's A row, scattered into slot order; each lane
     // zeroes its own padding slots (never a scatter target)
     stage_scatter(Ac, a.dst, nnz, sl, Lc, live, [&](int t, double v) { Abase[t] = v; });
-    zero_padding(Abase, a.padfrom, a.L, Lc, sl);
+    zero_padding(Abase, a.pads, a.npads, a.L, sl, Lc);
   }
   // pad rows of the product vectors are never written by the SpMV
   for (int i = n + sl; i < E * Lc; i += Lc) {
@@ -279,7 +273,10 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   }
   __syncwarp();
 
-  double r[E], p[E], s[E];
+  // r also holds s = r - alpha v between the half steps, and the true residual
+  // at the end; what a segment that no longer iterates keeps in r, p and the
+  // scalars is never read
+  double r[E], p[E];
   double bb;
   {
     double acc[1] = {0.0};
@@ -289,12 +286,11 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
       const bool v = live && i < n;
       const double bi = v ? (SRC == kSrcNewton ? nrh[i] : __ldg(a.b + (size_t)c * n + i)) : 0.0;
       const double d = v ? (ASMEM ? Abase[__ldg(a.dslot + i)]
-                               : __ldg(Ac + __ldg(a.src + __ldg(a.dslot + i)))) : 0.0;
+                               : __ldg(Ac + __ldg(a.dentry + i))) : 0.0;
       dvs[e] = v ? (!is_zero_bits(d) ? recip64(d) : 1.0) : 0.0;
       xv[e] = (v && a.x0_given) ? a.x[(size_t)c * n + i] : 0.0;
       r[e] = bi;
       p[e] = 0.0;
-      s[e] = 0.0;
       acc[0] = fma(bi, bi, acc[0]);
     }
     bb = ssum1<LC>(acc[0], Lc);
@@ -341,12 +337,8 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
       pass0 = false;
       if (restart) {
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-          rhs[e] = r[e];
-          p[e] = 0.0;
-        }
+        for (int e = 0; e < E; ++e) rhs[e] = r[e];
         rho = acc[0];
-        rho_prev = alpha = omega = 1.0;
         broke = nonfin = false;
         fin = true;
         // a restart follows a failed true-residual test: always iterate
@@ -355,6 +347,9 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
         first = false;
       }
     }
+    // The segments active in a pass all (re)started at its head, so its first
+    // iteration has p = r (beta times zero otherwise).
+    bool head = true;
     while (__any_sync(kFull, active)) {
       if (active) {
         if (it >= a.maxit) {
@@ -367,14 +362,19 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
           active = false;
         }
       }
-      // p = r + beta (p - omega v); the bracket is kept in p
-      const double beta = (rho * alpha) * recip64s(rho_prev * omega);
+      // p = r + beta (p - omega v), v of the iteration before
+      if (head) {
+        head = false;
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int i = sl + e * Lc;
-        if (active) p[e] = fma(beta, p[e], r[e]);
-        gs[i] = dvs[e] * p[e];
+        for (int e = 0; e < E; ++e) p[e] = r[e];
+      } else {
+        const double beta = (rho * alpha) * recip64s(rho_prev * omega);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          p[e] = fma(beta, fma(-omega, o1[sl + e * Lc], p[e]), r[e]);
       }
+#pragma unroll
+      for (int e = 0; e < E; ++e) gs[sl + e * Lc] = dvs[e] * p[e];
       __syncwarp();
       SPMV(o1);  // v = A p^
       __syncwarp();
@@ -395,34 +395,37 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
           active = false;
         }
       }
-      const double al = rho * recip64s(sg[0]);
-      if (active) alpha = al;
+      alpha = rho * recip64s(sg[0]);
+      double q0 = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int i = sl + e * Lc;
-        if (active) {
-          xv[e] = fma(al, gs[i], xv[e]);
-          s[e] = fma(-al, o1[i], r[e]);
-        }
-        gs[i] = dvs[e] * s[e];
+        if (active) xv[e] = fma(alpha, gs[i], xv[e]);
+        r[e] = fma(-alpha, o1[i], r[e]);  // s
+        q0 = fma(r[e], r[e], q0);
       }
+      q0 = ssum1<LC>(q0, Lc);
+      // Converged on the half step (x holds alpha p^).  Tested before the
+      // second product, which about half of all cells then never need in
+      // their last iteration.
+      if (active && le_nonneg(q0, thr)) active = false;
+      if (!__any_sync(kFull, active)) break;
+#pragma unroll
+      for (int e = 0; e < E; ++e) gs[sl + e * Lc] = dvs[e] * r[e];
       __syncwarp();
       SPMV(o2);  // t = A s^
       __syncwarp();
-      double q0 = 0.0, q1 = 0.0, q2 = 0.0;
+      double q1 = 0.0, q2 = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const double t = o2[sl + e * Lc];
-        q0 = fma(s[e], s[e], q0);
-        q1 = fma(t, s[e], q1);
+        q1 = fma(t, r[e], q1);
         q2 = fma(t, t, q2);
       }
-      ssum3<LC>(q0, q1, q2, Lc);
+      ssum2<LC>(q1, q2, Lc);
       bool full = false;
       if (active) {
-        if (le_nonneg(q0, thr)) {
-          active = false;  // converged on the half step (x live alpha p^)
-        } else if (!is_finite_bits(q1) || !is_finite_bits(q2)) {
+        if (!is_finite_bits(q1) || !is_finite_bits(q2)) {
           nonfin = true;
           active = false;
         } else if (is_zero_bits(q2)) {
@@ -432,20 +435,13 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
           full = true;
         }
       }
-      const double om = q1 * recip64s(q2);
-      if (full) omega = om;
-#pragma unroll
-      for (int e = 0; e < E; ++e) {
-        const int i = sl + e * Lc;
-        if (full) {
-          xv[e] = fma(om, gs[i], xv[e]);
-          r[e] = fma(-om, o2[i], s[e]);
-          p[e] = fma(-om, o1[i], p[e]);
-        }
-      }
+      omega = q1 * recip64s(q2);
       double hr = 0.0, rr = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
+        const int i = sl + e * Lc;
+        if (full) xv[e] = fma(omega, gs[i], xv[e]);
+        r[e] = fma(-omega, o2[i], r[e]);
         hr = fma(rhs[e], r[e], hr);
         rr = fma(r[e], r[e], rr);
       }
@@ -454,14 +450,13 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
         nbreak = 0;
         if (le_nonneg(rr, thr)) {
           active = false;
-        } else if (is_zero_bits(om)) {
+        } else if (is_zero_bits(omega)) {
           broke = true;
           active = false;
-        } else {
-          rho_prev = rho;
-          rho = hr;
         }
       }
+      rho_prev = rho;
+      rho = hr;
     }
     // ---- true residual of the segments that stopped iterating
 #pragma unroll
@@ -474,8 +469,8 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
     for (int e = 0; e < E; ++e) {
       const int i = sl + e * Lc;
       const double bi = (live && i < n) ? (SRC == kSrcNewton ? nrh[i] : __ldg(a.b + (size_t)c * n + i)) : 0.0;
-      s[e] = bi - o1[i];  // s holds the true residual here
-      rt2[0] = fma(s[e], s[e], rt2[0]);
+      r[e] = bi - o1[i];
+      rt2[0] = fma(r[e], r[e], rt2[0]);
     }
     rt2[0] = ssum1<LC>(rt2[0], Lc);
     if (fin) {
@@ -490,9 +485,7 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
       } else if (broke && ++nbreak >= 2) {
         st = CAMP_CELL_BREAKDOWN;
       } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[e] = s[e];
-        restart = true;
+        restart = true;  // from the true residual
       }
     }
     if (!__any_sync(kFull, restart)) break;
@@ -524,106 +517,96 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
 
 // Plain launch: one mechanism, the SpMV schedule in shared memory, groups of
 // k cells taken by warps from the dynamic queue (or a grid-stride loop).
-template <int E, int SRC>
+// LC: lanes per cell at compile time (0: a.Lc).  TK: which tickets the launch
+// has (the plain solve at 16 lanes only; see WarpArgs::single_from).  Each
+// combination is a kernel of its own: one kernel holding all of them spilled
+// 520 bytes a thread at 5 rows per lane, where each alone spills 8 at most.
+template <int E, int SRC, int LC, int TK>
 __device__ __forceinline__ void plain_launch_body(const WarpArgs &a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SchedWord *sch_s = reinterpret_cast<SchedWord *>(smem_raw);
-  const int nsch = a.L * a.Lc;
-  for (int i = threadIdx.x; i < nsch; i += blockDim.x) sch_s[i] = a.sched[i];
-  __syncthreads();
+  const int Lc = LC ? LC : a.Lc, k = LC ? 32 / LC : a.k;
+  const int nsch = a.L * Lc;
+  if constexpr (TK != kTicketsOne) {
+    for (int i = threadIdx.x; i < nsch; i += blockDim.x) sch_s[i] = a.sched[i];
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   double *wbase = reinterpret_cast<double *>(smem_raw + sched_smem_bytes(nsch)) +
-                  (size_t)warp * a.k * a.segStride;
-  const SchedWord *sch = sch_s + (lane & (a.Lc - 1));
+                  (size_t)warp * k * a.segStride;
   const int warps_total = gridDim.x * (blockDim.x >> 5);
   if (a.ord_ws)
     order_prologue<SRC != kSrcStaged>(a, reinterpret_cast<int *>(smem_raw + sched_smem_bytes(nsch)));
-  auto run = [&](auto lc) {
-    constexpr int LC = decltype(lc)::value;
-    if (!a.queue) {
-      for (int g = blockIdx.x * (blockDim.x >> 5) + warp; g < a.ngroups; g += warps_total)
-        solve_group<E, SRC, LC>(a, g, wbase, sch);
-      return;
+  if (!a.queue) {
+    for (int g = blockIdx.x * (blockDim.x >> 5) + warp; g < a.ngroups; g += warps_total)
+      solve_group<E, SRC, LC>(a, g, wbase, sch_s);
+    return;
+  }
+  // dynamic assignment: warps take the next group until none is left (an
+  // ordered launch first gives every warp one group of a stratified wave).
+  const bool strat = a.order && a.ord_stride == 0 && a.ord_wave > 0;
+  bool first = strat;
+  for (;;) {
+    unsigned g = 0;
+    if (first) {
+      first = false;
+      const unsigned B = gridDim.x, b = blockIdx.x, w = (unsigned)warp;
+      g = w * B + ((w & 1u) ? B - 1u - b : b);
+    } else {
+      if (lane == 0) g = atomicAdd(a.queue, 1u);
+      g = __shfl_sync(kFull, g, 0);
+      if (strat) g += (unsigned)a.ord_wave;
+      if (g >= (unsigned)a.ngroups) break;
+      if (a.order && a.ord_stride && g < (unsigned)a.ord_wave)
+        g = (unsigned)((unsigned long long)g * (unsigned)a.ord_stride % (unsigned)a.ord_wave);
     }
-    // dynamic assignment: warps take the next group until none is left (an
-    // ordered launch first gives every warp one group of a stratified wave).
-    // The steps of take_group / await_order_entries, written out: built from
-    // those helpers this kernel ran its first-wave groups far slower (272
-    // against 212 us at 80 species x 10,000 cells).
-    const bool strat = a.order && a.ord_stride == 0 && a.ord_wave > 0;
-    bool first = strat;
-    for (;;) {
-      unsigned g = 0;
-      if (first) {
-        first = false;
-        const unsigned B = gridDim.x, b = blockIdx.x, w = (unsigned)warp;
-        g = w * B + ((w & 1u) ? B - 1u - b : b);
-      } else {
-        if (lane == 0) g = atomicAdd(a.queue, 1u);
-        g = __shfl_sync(kFull, g, 0);
-        if (strat) g += (unsigned)a.ord_wave;
-        if (g >= (unsigned)a.ngroups) break;
-        if (a.order && a.ord_stride && g < (unsigned)a.ord_wave)
-          g = (unsigned)((unsigned long long)g * (unsigned)a.ord_stride % (unsigned)a.ord_wave);
+    if constexpr (TK != kTicketsPack) {
+      if (TK == kTicketsOne || (int)g >= a.single_from) {
+        // a single-cell ticket: one cell on all 32 lanes (warp_single.cuh)
+        const int ps = 2 * a.single_from + ((int)g - a.single_from);
+        const bool one = a.ord_ws && lane == 0 && ps < a.cells;
+        if (one) wait_order_entry(a.order + ps, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
+        __syncwarp();
+        solve_single<E>(a, ps, wbase);
+        if (one) a.ord_out[ps] = 0;
+        continue;
       }
-      if constexpr (SRC == kSrcStaged && LC == 16 && E <= kRegVecMaxE) {
-        if (a.sched2 && (int)g >= a.single_from) {
-          // a single-cell ticket: one cell on all 32 lanes (warp_single.cuh)
-          const int ps = 2 * a.single_from + ((int)g - a.single_from);
-          const bool one = a.ord_ws && lane == 0 && ps < a.cells;
-          if (one) wait_order_entry(a.order + ps, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
-          __syncwarp();
-          solve_single<E>(a, ps, wbase);
-          if (one) a.ord_out[ps] = 0;
-          continue;
-        }
-      }
+    }
+    if constexpr (TK != kTicketsOne) {
       // in-launch ordering: wait for this group's order entries, solve,
       // then clear them
-      const int p = (int)g * (LC ? 32 / LC : a.k) + lane;
-      const bool mine = a.ord_ws && lane < (LC ? 32 / LC : a.k) && p < a.cells;
+      const int p = (int)g * k + lane;
+      const bool mine = a.ord_ws && lane < k && p < a.cells;
       if (mine) wait_order_entry(a.order + p, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
       __syncwarp();
-      solve_group<E, SRC, LC>(a, (int)g, wbase, sch);
+      solve_group<E, SRC, LC>(a, (int)g, wbase, sch_s);
       if (mine) a.ord_out[p] = 0;
     }
-  };
-  // The arrangements the automatic choice makes for 21..160 rows (3 to 5 rows
-  // per lane on 8, 16 or 32 lanes) run code with Lc fixed at compile time:
-  // constant strides fold into the shared-memory addressing.
-  if constexpr (E >= 3 && E <= kRegVecMaxE) {
-    if (a.Lc == 16) run(std::integral_constant<int, 16>());
-    else if (a.Lc == 32) run(std::integral_constant<int, 32>());
-    else if (a.Lc == 8) run(std::integral_constant<int, 8>());
-    else run(std::integral_constant<int, 0>());
-  } else {
-    run(std::integral_constant<int, 0>());
   }
-  if (!a.queue) return;
   // the last warp resets the queue and the ordering workspace (and, after a
   // time-out of the ordering, marks the launch's cells invalid)
   finish_queue(a, true, warps_total, lane);
 }
 
-template <int E>
-__global__ void __launch_bounds__(256, CAMP_WARP_MINB)
-    warp_bicgstab_kernel(const WarpArgs a) {
-  plain_launch_body<E, kSrcStaged>(a);
+template <int E, int LC, int TK>
+__global__ void CAMP_WARP_BOUNDS
+    warp_bicgstab_kernel(const __grid_constant__ WarpArgs a) {
+  plain_launch_body<E, kSrcStaged, LC, TK>(a);
 }
 
 // Device Newton corrector of the implicit step around the assembly + solve.
-template <int E>
-__global__ void __launch_bounds__(256, CAMP_WARP_MINB)
-    newton_bicgstab_kernel(const WarpArgs a) {
-  plain_launch_body<E, kSrcNewton>(a);
+template <int E, int LC>
+__global__ void CAMP_WARP_BOUNDS
+    newton_bicgstab_kernel(const __grid_constant__ WarpArgs a) {
+  plain_launch_body<E, kSrcNewton, LC, kTicketsPack>(a);
 }
 
 // Fused Jacobian assembly and solve (A = I - gamma J(conc) built per cell).
-template <int E>
-__global__ void __launch_bounds__(256, CAMP_WARP_MINB)
-    assemble_bicgstab_kernel(const WarpArgs a) {
-  plain_launch_body<E, kSrcAssembled>(a);
+template <int E, int LC>
+__global__ void CAMP_WARP_BOUNDS
+    assemble_bicgstab_kernel(const __grid_constant__ WarpArgs a) {
+  plain_launch_body<E, kSrcAssembled, LC, kTicketsPack>(a);
 }
 
 // Persistent launch over several mechanisms (uneven batching): every warp
@@ -632,7 +615,7 @@ __global__ void __launch_bounds__(256, CAMP_WARP_MINB)
 // largest cells first, so the long items start early and the short ones fill
 // the tail.  The only wait is the atomic increment: no spin, no barrier.
 template <int E, bool ASMEM>
-__global__ void __launch_bounds__(256, CAMP_WARP_MINB)
+__global__ void CAMP_WARP_BOUNDS
     batch_bicgstab_kernel(const __grid_constant__ BatchArgs b) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
@@ -646,8 +629,7 @@ __global__ void __launch_bounds__(256, CAMP_WARP_MINB)
     int m = 0;
     while (m + 1 < b.nmech && item >= (unsigned)b.item_begin[m + 1]) ++m;
     const WarpArgs &a = b.m[m];
-    const SchedWord *sch = a.sched + (lane & (a.Lc - 1));
-    solve_group<E, ASMEM ? kSrcStaged : kSrcGlobal>(a, (int)item - b.item_begin[m], wbase, sch);
+    solve_group<E, ASMEM ? kSrcStaged : kSrcGlobal>(a, (int)item - b.item_begin[m], wbase, a.sched);
   }
 }
 

@@ -52,13 +52,12 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
                                (unsigned)a.cells - 1u)
                     : pos;
   const double *Ac = a.A + (size_t)(has ? c : 0) * nnz;
-  const SchedWord *sch = a.sched2 + lane;
-  const double *Asl = Abase + lane;
+  const unsigned gsa = smem_addr(gs);
   // row of register slot j (the upper lanes' spare slot, when E16 is odd,
   // maps to row v: it is never read or written, and no address it could
   // form leaves the region)
   auto row = [&](int j) { return v + 16 * (h ? (j < E16 - E0 ? E0 + j : 0) : j); };
-  auto spmv = [&](double *out) { seg_spmv(sch, a.L2, 32, Asl, gs, out); };
+  auto spmv = [&](double *out) { seg_spmv(a.sched2, a.ends2, a.L2, 32, lane, Abase, gsa, smem_addr(out)); };
   // the chained dot products: stage one on the lower lanes, the hand-off,
   // stage two on the upper lanes, then the exact sum over the warp
 #define CHAIN(acc, X, Y)                                             \
@@ -78,7 +77,7 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
 
   // ---- stage the cell's matrix values in split-slot order
   stage_scatter(Ac, a.dst2, nnz, lane, 32, live, [&](int t, double x) { Abase[t] = x; });
-  zero_padding(Abase, a.padfrom2, a.L2, 32, lane);
+  zero_padding(Abase, a.pads2, a.npads2, a.L2, lane, 32);
   // pad rows of the product vectors are never written by the SpMV
   for (int i = n + lane; i < 16 * E16; i += 32) {
     o1[i] = 0.0;
@@ -86,7 +85,7 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
   }
   __syncwarp();
 
-  double r[E0], p[E0], s[E0];
+  double r[E0], p[E0];  // r also holds s and the true residual, as in solve_group
   double bb;
   {
     double acc = 0.0;
@@ -100,7 +99,6 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
       xv[j] = (ok && a.x0_given) ? a.x[(size_t)c * n + i] : 0.0;
       r[j] = bi;
       p[j] = 0.0;
-      s[j] = 0.0;
       rhs[j] = 0.0;
     }
     CHAIN(acc, r[j], r[j]);
@@ -149,12 +147,8 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
       pass0 = false;
       if (restart) {
 #pragma unroll
-        for (int j = 0; j < E0; ++j) {
-          rhs[j] = r[j];
-          p[j] = 0.0;
-        }
+        for (int j = 0; j < E0; ++j) rhs[j] = r[j];
         rho = acc;
-        rho_prev = alpha = omega = 1.0;
         broke = nonfin = false;
         fin = true;
         active = first ? !le_nonneg(acc, thr) : true;
@@ -162,6 +156,7 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
         first = false;
       }
     }
+    bool head = true;  // the pass's first iteration: p = r
     while (__any_sync(kFull, active)) {
       if (active) {
         if (it >= a.maxit) {
@@ -174,13 +169,20 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
           active = false;
         }
       }
-      // p = r + beta (p - omega v); the bracket is kept in p
-      const double beta = (rho * alpha) * recip64s(rho_prev * omega);
+      // p = r + beta (p - omega v), v of the iteration before
+      if (head) {
+        head = false;
 #pragma unroll
-      for (int j = 0; j < E0; ++j) {
-        if (active) p[j] = fma(beta, p[j], r[j]);
-        if (j < EJ) gs[row(j)] = dvs[j] * p[j];
+        for (int j = 0; j < E0; ++j) p[j] = r[j];
+      } else {
+        const double beta = (rho * alpha) * recip64s(rho_prev * omega);
+#pragma unroll
+        for (int j = 0; j < E0; ++j)
+          if (j < EJ) p[j] = fma(beta, fma(-omega, o1[row(j)], p[j]), r[j]);
       }
+#pragma unroll
+      for (int j = 0; j < E0; ++j)
+        if (j < EJ) gs[row(j)] = dvs[j] * p[j];
       __syncwarp();
       spmv(o1);  // v = A p^
       __syncwarp();
@@ -197,23 +199,28 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
           active = false;
         }
       }
-      const double al = rho * recip64s(sg);
-      if (active) alpha = al;
+      alpha = rho * recip64s(sg);
 #pragma unroll
       for (int j = 0; j < E0; ++j) {
         if (j < EJ) {
           const int i = row(j);
-          if (active) {
-            xv[j] = fma(al, gs[i], xv[j]);
-            s[j] = fma(-al, o1[i], r[j]);
-          }
-          gs[i] = dvs[j] * s[j];
+          if (active) xv[j] = fma(alpha, gs[i], xv[j]);
+          r[j] = fma(-alpha, o1[i], r[j]);  // s
         }
       }
+      double q0 = 0.0;
+      CHAIN(q0, r[j], r[j]);
+      q0 = seg_sum_exact_redux<1>(q0);
+      // converged on the half step (x holds alpha p^), before the second product
+      if (active && le_nonneg(q0, thr)) active = false;
+      if (!__any_sync(kFull, active)) break;
+#pragma unroll
+      for (int j = 0; j < E0; ++j)
+        if (j < EJ) gs[row(j)] = dvs[j] * r[j];
       __syncwarp();
       spmv(o2);  // t = A s^
       __syncwarp();
-      double q0 = 0.0, q1 = 0.0, q2 = 0.0;
+      double q1 = 0.0, q2 = 0.0;
       {
         double t[E0];
 #pragma unroll
@@ -221,32 +228,25 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
 #pragma unroll
         for (int j = 0; j < E0; ++j)
           if (h == 0) {
-            q0 = fma(s[j], s[j], q0);
-            q1 = fma(t[j], s[j], q1);
+            q1 = fma(t[j], r[j], q1);
             q2 = fma(t[j], t[j], q2);
           }
-        q0 = split_handoff(q0, h, v);
         q1 = split_handoff(q1, h, v);
         q2 = split_handoff(q2, h, v);
 #pragma unroll
         for (int j = 0; j < E0; ++j)
           if (h == 1 && j < EJ) {
-            q0 = fma(s[j], s[j], q0);
-            q1 = fma(t[j], s[j], q1);
+            q1 = fma(t[j], r[j], q1);
             q2 = fma(t[j], t[j], q2);
           }
-        q0 = h ? q0 : 0.0;
         q1 = h ? q1 : 0.0;
         q2 = h ? q2 : 0.0;
       }
-      q0 = seg_sum_exact_redux<1>(q0);
       q1 = seg_sum_exact_redux<1>(q1);
       q2 = seg_sum_exact_redux<1>(q2);
       bool full = false;
       if (active) {
-        if (le_nonneg(q0, thr)) {
-          active = false;  // converged on the half step (x live alpha p^)
-        } else if (!is_finite_bits(q1) || !is_finite_bits(q2)) {
+        if (!is_finite_bits(q1) || !is_finite_bits(q2)) {
           nonfin = true;
           active = false;
         } else if (is_zero_bits(q2)) {
@@ -256,17 +256,14 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
           full = true;
         }
       }
-      const double om = q1 * recip64s(q2);
-      if (full) omega = om;
+      omega = q1 * recip64s(q2);
 #pragma unroll
-      for (int j = 0; j < E0; ++j) {
-        if (full && j < EJ) {
+      for (int j = 0; j < E0; ++j)
+        if (j < EJ) {
           const int i = row(j);
-          xv[j] = fma(om, gs[i], xv[j]);
-          r[j] = fma(-om, o2[i], s[j]);
-          p[j] = fma(-om, o1[i], p[j]);
+          if (full) xv[j] = fma(omega, gs[i], xv[j]);
+          r[j] = fma(-omega, o2[i], r[j]);
         }
-      }
       double hr = 0.0, rr = 0.0;
 #pragma unroll
       for (int j = 0; j < E0; ++j)
@@ -290,14 +287,13 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
         nbreak = 0;
         if (le_nonneg(rr, thr)) {
           active = false;
-        } else if (is_zero_bits(om)) {
+        } else if (is_zero_bits(omega)) {
           broke = true;
           active = false;
-        } else {
-          rho_prev = rho;
-          rho = hr;
         }
       }
+      rho_prev = rho;
+      rho = hr;
     }
     // ---- true residual
 #pragma unroll
@@ -311,9 +307,9 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
     for (int j = 0; j < E0; ++j) {
       const int i = row(j);
       const double bi = (live && j < EJ && i < n) ? __ldg(a.b + (size_t)c * n + i) : 0.0;
-      s[j] = j < EJ ? bi - o1[i] : 0.0;  // s holds the true residual here
+      r[j] = j < EJ ? bi - o1[i] : 0.0;
     }
-    CHAIN(rt2, s[j], s[j]);
+    CHAIN(rt2, r[j], r[j]);
     rt2 = seg_sum_exact_redux<1>(rt2);
     if (fin) {
       fin = false;
@@ -327,9 +323,7 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
       } else if (broke && ++nbreak >= 2) {
         st = CAMP_CELL_BREAKDOWN;
       } else {
-#pragma unroll
-        for (int j = 0; j < E0; ++j) r[j] = s[j];
-        restart = true;
+        restart = true;  // from the true residual
       }
     }
     if (!__any_sync(kFull, restart)) break;

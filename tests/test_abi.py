@@ -405,3 +405,65 @@ def test_split_schedule_with_many_rows_on_one_lane(lib):
     w2 = words.reshape(L.value, 32, 2)
     assert _rows_of_schedule(w16, L16, 16) == _rows_of_schedule(w2, L.value, 32)
     assert L.value <= L16
+
+
+def _aligned(lib, m, lc, split):
+    f = lib.camp_schedule_build_aligned
+    f.restype = ctypes.c_int
+    f.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int,
+                  ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.POINTER(ctypes.c_int)]
+    rp = np.ascontiguousarray(m.row_ptr, np.int32)
+    ci = np.ascontiguousarray(m.col_idx, np.int32)
+    L = ctypes.c_int()
+    lanes = 32 if split else lc
+    assert f(m.n, m.nnz, rp.ctypes.data, ci.ctypes.data, lc, split, None, 0, ctypes.byref(L)) == 0
+    words = np.zeros(2 * max(1, L.value * lanes), np.uint32)
+    assert f(m.n, m.nnz, rp.ctypes.data, ci.ctypes.data, lc, split, words.ctypes.data,
+             L.value * lanes, ctypes.byref(L)) == 0
+    return L.value, words[:2 * L.value * lanes].reshape(L.value, lanes, 2)
+
+
+@pytest.mark.parametrize("n,R", [(3, 4), (9, 14), (21, 50), (40, 90), (57, 140), (80, 200), (150, 400)])
+@pytest.mark.parametrize("lc,split", [(8, 0), (16, 0), (16, 1), (32, 0)])
+def test_aligned_layout_keeps_every_row_chain(lib, n, R, lc, split):
+    """The aligned layout gives every row exactly the entries, in exactly the
+    order, of its schedule (so each row's sum is the same chain of
+    multiply-adds), in no more slots per lane; padding inside a lane leads a
+    row and reads a column of that row, and the 80-row layout on 16 lanes ends
+    rows in at most a third of its slots."""
+    import synth
+    m = synth.make_mechanism(n, R, 40 + n)
+    if (n + lc - 1) // lc > 16:
+        pytest.skip("more rows per lane than the kernels take")
+    L0, w0 = _schedule(lib, "camp_schedule_build", m, lc)
+    L, w = _aligned(lib, m, lc, split)
+    if L == 0:
+        assert n < 21 or n > 5 * lc   # found for every automatic lane count above 20 rows
+        return
+    assert L <= (L0 if not split else (L0 + 1) // 2 + int(np.diff(m.row_ptr).max()))
+    lanes = 32 if split else lc
+    rows0 = _rows_of_schedule(w0, L0, lc)
+    rows = {}
+    ends = set()
+    for q in range(lanes):
+        cur, lead = [], []
+        for j in range(L):
+            src, w1 = int(w[j, q, 0]), int(w[j, q, 1])
+            col = w1 & 0x7FF
+            assert col < m.n
+            if src == 0xFFFFFFFF:
+                assert not w1 >> 31 and not cur, "padding only between rows"
+                lead.append(col)
+                continue
+            assert int(m.col_idx[src]) == col
+            cur.append(src)
+            if w1 >> 31:
+                row = (w1 >> 11) & 0x7FF
+                own = set(m.col_idx[m.row_ptr[row]:m.row_ptr[row + 1]].tolist())
+                assert set(lead) <= own
+                rows[row], cur, lead = cur, [], []
+                ends.add(j)
+        assert not cur
+    assert rows == rows0
+    if n == 80 and lc == 16 and not split:
+        assert len(ends) <= L // 3
