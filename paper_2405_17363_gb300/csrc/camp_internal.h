@@ -296,7 +296,6 @@ struct MixedArgs {
   const int *dst32;    // [nnz] place (word_pos) of each A entry in the FP32 copy
   const int *pads, *pads32;  // [npads] places of the padding slots in either copy
   int npads;
-  unsigned ends[kEndWords];
   const int *dslot32;  // [n] place (word_pos) of each row's diagonal entry
   double tol;
   int max_sweeps;

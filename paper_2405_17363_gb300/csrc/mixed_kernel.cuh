@@ -109,8 +109,8 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 #pragma unroll
         for (int e = 0; e < E; ++e) g64[sl + e * Lc] = xv[e];
         __syncwarp();
-        if (a.a64_smem) seg_spmv(sch, a.ends, a.L, Lc, sl, As, g64a, o64a);
-        else seg_spmv_gather(sch, a.ends, a.src, a.L, Lc, sl, Ac, g64a, o64a);
+        if (a.a64_smem) flat_spmv(sch, a.L, Lc, sl, As, g64a, o64a);
+        else flat_spmv_gather(sch, a.src, a.L, Lc, sl, Ac, g64a, o64a);
         __syncwarp();
       }
       double rr[1] = {0.0};
@@ -187,7 +187,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 #pragma unroll
         for (int e = 0; e < E; ++e) g32[sl + e * Lc] = dinv[e] * p[e];
         __syncwarp();
-        seg_spmvf(sch, a.L, Lc, sl, As32, g32a, o1a);
+        flat_spmvf(sch, a.L, Lc, sl, As32, g32a, o1a);
         __syncwarp();
         if (act) ++it;
         float sg[1] = {0.0f};
@@ -211,7 +211,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 #pragma unroll
         for (int e = 0; e < E; ++e) g32[sl + e * Lc] = dinv[e] * rf[e];
         __syncwarp();
-        seg_spmvf(sch, a.L, Lc, sl, As32, g32a, o2a);
+        flat_spmvf(sch, a.L, Lc, sl, As32, g32a, o2a);
         __syncwarp();
         float qt[2] = {0.0f, 0.0f};
 #pragma unroll

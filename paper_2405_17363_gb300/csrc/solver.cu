@@ -573,15 +573,17 @@ void free_view(View &v) {
 }
 
 // A launch's schedule arguments.
+void set_ends(WarpArgs &a, const Slots &S) { memcpy(a.ends, S.ends, sizeof a.ends); }
+void set_ends(MixedArgs &, const Slots &) {}
 template <class Args>
 void set_slots(Args &a, const Slots &S) {
+  set_ends(a, S);
   a.L = S.L;
   a.sched = S.d_words;
   a.src = S.d_src;
   a.dst = S.d_dst;
   a.pads = S.d_pads;
   a.npads = S.npads;
-  memcpy(a.ends, S.ends, sizeof a.ends);
 }
 
 int ilog2(int v) {

@@ -284,17 +284,20 @@ __device__ __forceinline__ void seg_sumf(float (&v)[NV], int Lc) {
   }
 }
 
-// The FP32 product (A32 in slot order, word_pos places), with a row end in
-// every slot (a predicated store and a select, no branch): an FP32 chain is
-// short, so issue slots bound it, and the branches of spmv_slots cost more
-// than they save (150 species x 100,000 cells: 1,983 us against 2,195).
-__device__ __forceinline__ void seg_spmvf(const SchedWord *__restrict__ sch, int L, int Lc, int sl,
-                                          const float *__restrict__ As, unsigned gs, unsigned os) {
+// The same product with a row end in every slot (a predicated store and a
+// select, no branch), as the refinement kernel runs it on the schedule as
+// built: an FP32 chain is short, so issue slots and shared-memory wavefronts
+// bound that kernel, and the branches of spmv_slots and the bank conflicts of
+// aligned rows cost it more than they save (150 species x 100,000 cells:
+// 1,983 us against 2,195).  block(b, av): the A values of slots 4b .. 4b+3;
+// one(j): that of slot j past the last whole block.
+template <class T, class Block, class One>
+__device__ __forceinline__ void spmv_flat(const SchedWord *__restrict__ sch, int L, int Lc, int sl,
+                                          Block block, One one, unsigned gs, unsigned os) {
   const uint4 *s4 = reinterpret_cast<const uint4 *>(sch) + sl;
-  const float4 *A4 = reinterpret_cast<const float4 *>(As) + sl;
-  float acc = 0.0f;
+  T acc = T(0);
   const int nb = L >> 2;
-  auto step = [&](unsigned w, float av, float xv) {
+  auto step = [&](unsigned w, T av, T xv) {
     acc = fma_t(av, xv, acc);
     slot_end(w, acc, os);
   };
@@ -302,18 +305,18 @@ __device__ __forceinline__ void seg_spmvf(const SchedWord *__restrict__ sch, int
     uint4 w = *s4;
 #pragma unroll 1
     for (int b = 0;;) {
-      float x0, x1, x2, x3;
-      lds(x0, slot_col_addr<float>(w.x, gs));
-      lds(x1, slot_col_addr<float>(w.y, gs));
-      lds(x2, slot_col_addr<float>(w.z, gs));
-      lds(x3, slot_col_addr<float>(w.w, gs));
-      const float4 av = A4[b * Lc];
+      T av[4], x0, x1, x2, x3;
+      lds(x0, slot_col_addr<T>(w.x, gs));
+      lds(x1, slot_col_addr<T>(w.y, gs));
+      lds(x2, slot_col_addr<T>(w.z, gs));
+      lds(x3, slot_col_addr<T>(w.w, gs));
+      block(b, av);
       uint4 wn = w;
       if (++b < nb) wn = s4[b * Lc];
-      step(w.x, av.x, x0);
-      step(w.y, av.y, x1);
-      step(w.z, av.z, x2);
-      step(w.w, av.w, x3);
+      step(w.x, av[0], x0);
+      step(w.y, av[1], x1);
+      step(w.z, av[2], x2);
+      step(w.w, av[3], x3);
       if (b == nb) break;
       w = wn;
     }
@@ -322,10 +325,50 @@ __device__ __forceinline__ void seg_spmvf(const SchedWord *__restrict__ sch, int
   for (int u = 0; u < 3; ++u)
     if ((L & 3) > u) {
       const unsigned w = sch[(4 * nb + u) * Lc + sl];
-      float x;
-      lds(x, slot_col_addr<float>(w, gs));
-      step(w, As[(4 * nb + u) * Lc + sl], x);
+      T x;
+      lds(x, slot_col_addr<T>(w, gs));
+      step(w, one(4 * nb + u), x);
     }
+}
+
+// FP32, A32 in slot order in shared memory (word_pos places).
+__device__ __forceinline__ void flat_spmvf(const SchedWord *__restrict__ sch, int L, int Lc, int sl,
+                                           const float *__restrict__ As, unsigned gs, unsigned os) {
+  const float4 *A4 = reinterpret_cast<const float4 *>(As) + sl;
+  spmv_flat<float>(
+      sch, L, Lc, sl,
+      [&](int b, float *av) {
+        const float4 p = A4[b * Lc];
+        av[0] = p.x; av[1] = p.y; av[2] = p.z; av[3] = p.w;
+      },
+      [&](int j) { return As[j * Lc + sl]; }, gs, os);
+}
+// FP64, A in shared memory (pair_pos places), or read from global memory
+// through the slots' source entries.
+__device__ __forceinline__ void flat_spmv(const SchedWord *__restrict__ sch, int L, int Lc, int sl,
+                                          const double *__restrict__ As, unsigned gs, unsigned os) {
+  const double2 *A2 = reinterpret_cast<const double2 *>(As) + sl;
+  spmv_flat<double>(
+      sch, L, Lc, sl,
+      [&](int b, double *av) {
+        const double2 p = A2[(2 * b) * Lc], q = A2[(2 * b + 1) * Lc];
+        av[0] = p.x; av[1] = p.y; av[2] = q.x; av[3] = q.y;
+      },
+      [&](int j) { return As[pair_pos(j, sl, L, Lc)]; }, gs, os);
+}
+__device__ __forceinline__ void flat_spmv_gather(const SchedWord *__restrict__ sch,
+                                                 const int *__restrict__ src, int L, int Lc, int sl,
+                                                 const double *__restrict__ Ag, unsigned gs,
+                                                 unsigned os) {
+  const int4 *s4 = reinterpret_cast<const int4 *>(src) + sl;
+  auto value = [&](int k) { return k >= 0 ? __ldg(Ag + k) : 0.0; };
+  spmv_flat<double>(
+      sch, L, Lc, sl,
+      [&](int b, double *av) {
+        const int4 k = __ldg(s4 + b * Lc);
+        av[0] = value(k.x); av[1] = value(k.y); av[2] = value(k.z); av[3] = value(k.w);
+      },
+      [&](int j) { return value(__ldg(src + j * Lc + sl)); }, gs, os);
 }
 
 // FP64 -> FP32 conversion, round to nearest even, entirely on the integer
@@ -410,6 +453,32 @@ __device__ __forceinline__ double recip64(double d) { return recip64n<2>(d); }
 // about 2^-44; x and r are updated with the same scalar, so they stay
 // consistent and the true-residual test still decides convergence.
 __device__ __forceinline__ double recip64s(double d) { return recip64n<1>(d); }
+
+// A high word H such that every v whose |v| has a larger one satisfies
+// v^2 > thr, also after rounding: the high word of an upper bound of
+// sqrt(thr) (the fraction rounded up to FP32, an approximate FP32 square root,
+// 2^-18 on top for its error).  Then a sum of squares that contains v^2, as a
+// chain of multiply-adds from zero and the exact sum of the chains, is above
+// thr too (each only grows, and rounding is monotone), so the convergence test
+// ||r||^2 <= thr needs neither while one entry of r stands out: near
+// convergence alone it is evaluated.  Saves 10 of 153 FP64 instructions and
+// two of six exact sums per iteration.  thr outside [2^-900, 2^900]: no v.
+__device__ __forceinline__ unsigned sqrt_bound_hi(double thr) {
+  const unsigned hi = (unsigned)__double2hiint(thr), lo = (unsigned)__double2loint(thr);
+  const int ed = (int)(hi >> 20);
+  const int e = ed - 1023, odd = e & 1;
+  float t = __uint_as_float((0x3f800000u | (hi & 0xfffffu) << 3 | lo >> 29) + 1u);
+  t = odd ? t + t : t;
+  asm("sqrt.approx.ftz.f32 %0, %0;" : "+f"(t));
+  t = fmaf(t, 0x1p-18f, t);
+  const unsigned tb = __float_as_uint(t);
+  const unsigned H = (unsigned)(1023 + (e - odd) / 2 + (int)(tb >> 23) - 127) << 20 |
+                     ((tb >> 3) & 0xfffffu);
+  return ed >= 123 && ed <= 1923 ? H : 0x7fffffffu;
+}
+__device__ __forceinline__ unsigned abs_hi(double v) {
+  return (unsigned)__double2hiint(v) & 0x7fffffffu;
+}
 
 // Sum of v over the Lc lanes of each segment on the integer pipe.  Every
 // term m 2^(e-1075) (53-bit integer m) is aligned to the segment's largest

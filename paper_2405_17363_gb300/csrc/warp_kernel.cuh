@@ -296,6 +296,21 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
     bb = ssum1<LC>(acc[0], Lc);
   }
   const double thr = (tol * tol) * bb;  // (tol ||b||)^2
+  const unsigned far_hi = sqrt_bound_hi(thr);
+  const unsigned segm = Lc == 32 ? kFull : ((1u << (Lc & 31)) - 1u) << (seg * Lc);
+  // whether ||r||^2 > thr shows from one entry (the same for a segment's lanes)
+  auto stands_out = [&]() {
+    unsigned m = 0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) m = max(m, abs_hi(r[e]));
+    return (__ballot_sync(kFull, m > far_hi) & segm) != 0;
+  };
+  auto norm2 = [&]() {
+    double acc = 0.0;
+#pragma unroll
+    for (int e = 0; e < E; ++e) acc = fma(r[e], r[e], acc);
+    return ssum1<LC>(acc, Lc);
+  };
   int nbreak = 0;
   bool done = !live;
   if (live) {
@@ -326,23 +341,17 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   double rho = 1.0, rho_prev = 1.0, alpha = 1.0, omega = 1.0;
   for (;;) {
     {  // (re)start from the current residual r
-      double acc[1] = {0.0};
-      if (pass0 && !a.x0_given) {
-        acc[0] = bb;  // r = b: the same chain and exact sum as ||b||^2
-      } else {
-#pragma unroll
-        for (int e = 0; e < E; ++e) acc[0] = fma(r[e], r[e], acc[0]);
-        acc[0] = ssum1<LC>(acc[0], Lc);
-      }
+      // r = b: the same chain and exact sum as ||b||^2
+      const double rr = (pass0 && !a.x0_given) ? bb : norm2();
       pass0 = false;
       if (restart) {
 #pragma unroll
         for (int e = 0; e < E; ++e) rhs[e] = r[e];
-        rho = acc[0];
+        rho = rr;
         broke = nonfin = false;
         fin = true;
         // a restart follows a failed true-residual test: always iterate
-        active = first ? !le_nonneg(acc[0], thr) : true;
+        active = first ? !le_nonneg(rr, thr) : true;
         restart = false;
         first = false;
       }
@@ -396,20 +405,20 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
         }
       }
       alpha = rho * recip64s(sg[0]);
-      double q0 = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int i = sl + e * Lc;
         if (active) xv[e] = fma(alpha, gs[i], xv[e]);
         r[e] = fma(-alpha, o1[i], r[e]);  // s
-        q0 = fma(r[e], r[e], q0);
       }
-      q0 = ssum1<LC>(q0, Lc);
-      // Converged on the half step (x holds alpha p^).  Tested before the
+      // Converged on the half step (x holds alpha p^)?  Tested before the
       // second product, which about half of all cells then never need in
       // their last iteration.
-      if (active && le_nonneg(q0, thr)) active = false;
-      if (!__any_sync(kFull, active)) break;
+      const bool far = stands_out();
+      if (__any_sync(kFull, active && !far)) {
+        if (le_nonneg(norm2(), thr)) active = false;
+        if (!__any_sync(kFull, active)) break;
+      }
 #pragma unroll
       for (int e = 0; e < E; ++e) gs[sl + e * Lc] = dvs[e] * r[e];
       __syncwarp();
@@ -436,19 +445,21 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
         }
       }
       omega = q1 * recip64s(q2);
-      double hr = 0.0, rr = 0.0;
+      double hr = 0.0;
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int i = sl + e * Lc;
         if (full) xv[e] = fma(omega, gs[i], xv[e]);
         r[e] = fma(-omega, o2[i], r[e]);
         hr = fma(rhs[e], r[e], hr);
-        rr = fma(r[e], r[e], rr);
       }
-      ssum2<LC>(hr, rr, Lc);
+      bool conv = false;
+      const bool far2 = stands_out();
+      if (__any_sync(kFull, full && !far2)) conv = le_nonneg(norm2(), thr);
+      hr = ssum1<LC>(hr, Lc);
       if (full) {
         nbreak = 0;
-        if (le_nonneg(rr, thr)) {
+        if (conv) {
           active = false;
         } else if (is_zero_bits(omega)) {
           broke = true;
@@ -464,18 +475,16 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
     __syncwarp();
     SPMV(o1);
     __syncwarp();
-    double rt2[1] = {0.0};
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int i = sl + e * Lc;
       const double bi = (live && i < n) ? (SRC == kSrcNewton ? nrh[i] : __ldg(a.b + (size_t)c * n + i)) : 0.0;
       r[e] = bi - o1[i];
-      rt2[0] = fma(r[e], r[e], rt2[0]);
     }
-    rt2[0] = ssum1<LC>(rt2[0], Lc);
+    const double rt2 = norm2();
     if (fin) {
       fin = false;
-      resid = sqrt(rt2[0] * recip64(bb));
+      resid = sqrt(rt2 * recip64(bb));
       if (nonfin || !is_finite_bits(resid)) {
         st = CAMP_CELL_NONFINITE;
       } else if (resid <= tol) {

@@ -105,6 +105,19 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
     bb = seg_sum_exact_redux<1>(acc);
   }
   const double thr = (tol * tol) * bb;  // (tol ||b||)^2
+  const unsigned far_hi = sqrt_bound_hi(thr);
+  auto stands_out = [&]() {  // ||r||^2 > thr shows from one entry
+    unsigned m = 0;
+#pragma unroll
+    for (int j = 0; j < E0; ++j)
+      if (j < EJ) m = max(m, abs_hi(r[j]));
+    return __any_sync(kFull, m > far_hi);
+  };
+  auto norm2 = [&]() {
+    double acc = 0.0;
+    CHAIN(acc, r[j], r[j]);
+    return seg_sum_exact_redux<1>(acc);
+  };
   int nbreak = 0;
   bool done = !live;
   if (live) {
@@ -137,21 +150,16 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
   double rho = 1.0, rho_prev = 1.0, alpha = 1.0, omega = 1.0;
   for (;;) {
     {  // (re)start from the current residual r
-      double acc = 0.0;
-      if (pass0 && !a.x0_given) {
-        acc = bb;  // r = b: the same chain and exact sum as ||b||^2
-      } else {
-        CHAIN(acc, r[j], r[j]);
-        acc = seg_sum_exact_redux<1>(acc);
-      }
+      // r = b: the same chain and exact sum as ||b||^2
+      const double rr = (pass0 && !a.x0_given) ? bb : norm2();
       pass0 = false;
       if (restart) {
 #pragma unroll
         for (int j = 0; j < E0; ++j) rhs[j] = r[j];
-        rho = acc;
+        rho = rr;
         broke = nonfin = false;
         fin = true;
-        active = first ? !le_nonneg(acc, thr) : true;
+        active = first ? !le_nonneg(rr, thr) : true;
         restart = false;
         first = false;
       }
@@ -208,12 +216,11 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
           r[j] = fma(-alpha, o1[i], r[j]);  // s
         }
       }
-      double q0 = 0.0;
-      CHAIN(q0, r[j], r[j]);
-      q0 = seg_sum_exact_redux<1>(q0);
       // converged on the half step (x holds alpha p^), before the second product
-      if (active && le_nonneg(q0, thr)) active = false;
-      if (!__any_sync(kFull, active)) break;
+      if (!stands_out()) {
+        if (le_nonneg(norm2(), thr)) active = false;
+        if (!__any_sync(kFull, active)) break;
+      }
 #pragma unroll
       for (int j = 0; j < E0; ++j)
         if (j < EJ) gs[row(j)] = dvs[j] * r[j];
@@ -264,28 +271,13 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
           if (full) xv[j] = fma(omega, gs[i], xv[j]);
           r[j] = fma(-omega, o2[i], r[j]);
         }
-      double hr = 0.0, rr = 0.0;
-#pragma unroll
-      for (int j = 0; j < E0; ++j)
-        if (h == 0) {
-          hr = fma(rhs[j], r[j], hr);
-          rr = fma(r[j], r[j], rr);
-        }
-      hr = split_handoff(hr, h, v);
-      rr = split_handoff(rr, h, v);
-#pragma unroll
-      for (int j = 0; j < E0; ++j)
-        if (h == 1 && j < EJ) {
-          hr = fma(rhs[j], r[j], hr);
-          rr = fma(r[j], r[j], rr);
-        }
-      hr = h ? hr : 0.0;
-      rr = h ? rr : 0.0;
+      double hr = 0.0;
+      CHAIN(hr, rhs[j], r[j]);
+      const bool conv = !stands_out() && le_nonneg(norm2(), thr);
       hr = seg_sum_exact_redux<1>(hr);
-      rr = seg_sum_exact_redux<1>(rr);
       if (full) {
         nbreak = 0;
-        if (le_nonneg(rr, thr)) {
+        if (conv) {
           active = false;
         } else if (is_zero_bits(omega)) {
           broke = true;
@@ -302,15 +294,13 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
     __syncwarp();
     spmv(o1);
     __syncwarp();
-    double rt2 = 0.0;
 #pragma unroll
     for (int j = 0; j < E0; ++j) {
       const int i = row(j);
       const double bi = (live && j < EJ && i < n) ? __ldg(a.b + (size_t)c * n + i) : 0.0;
       r[j] = j < EJ ? bi - o1[i] : 0.0;
     }
-    CHAIN(rt2, r[j], r[j]);
-    rt2 = seg_sum_exact_redux<1>(rt2);
+    const double rt2 = norm2();
     if (fin) {
       fin = false;
       resid = sqrt(rt2 * recip64(bb));
