@@ -316,12 +316,13 @@ struct MixedArgs {
   long long ord_wait;
 };
 // Shared-memory bytes per cell of the refinement kernel: FP32 A, FP64 A when
-// staged, two FP64 and three FP32 vectors, rounded to 16.
+// staged, and two FP64 vectors, whose space the three FP32 vectors of the
+// inner iteration share; rounded to 16.
 __host__ __device__ inline size_t mixed_cell_bytes(int segA, int segV, bool a64_smem) {
-  return ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)28 * segV + 15) & ~(size_t)15;
+  return ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)16 * segV + 15) & ~(size_t)15;
 }
 // a cooperative launch when a.ord_ws is set (grid at most SMs x occupancy)
 cudaError_t launch_mixed(int E, const MixedArgs &a, int warps_per_block,
                          int grid, size_t smem, cudaStream_t st);
-cudaError_t mixed_occupancy(int E, int warps_per_block, size_t smem, int *blocks);
+cudaError_t mixed_occupancy(int E, int Lc, int warps_per_block, size_t smem, int *blocks);
 }  // namespace camp

@@ -10,8 +10,9 @@
 // FP64 [segA] (otherwise the FP64 residual product reads A through L1 from
 // the cell's row in global memory, which the staging has just brought into
 // L2: it runs two or three times per cell, against tens of FP32 products, and
-// the smaller footprint lets more warps run), the FP64 product input/output
-// vectors [segV each] and three FP32 vectors [segV each].
+// the smaller footprint lets more warps run), and the FP64 product's input and
+// output vectors [segV each], whose space the inner iteration's three FP32
+// vectors take in turn.
 #pragma once
 #include "warp_common.cuh"
 
@@ -30,8 +31,6 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
   const int seg = LC ? lane / LC : lane >> a.log2Lc;
   const int sl = lane & (Lc - 1);
   const int n = a.n, nnz = a.nnz;
-  // bytes per cell: (12 or 4) segA + 16 segV + 12 segV (FP64 A when staged,
-  // FP32 A, 2 FP64 + 3 FP32 vectors)
   const size_t cellBytes = mixed_cell_bytes(a.segA, a.segV, a.a64_smem);
   unsigned char *wb = smem_raw + sched_smem_bytes(nsch) +
                       ((size_t)warp * a.k + seg) * cellBytes;
@@ -39,16 +38,13 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
   double *g64 = As + (a.a64_smem ? a.segA : 0);
   double *o64 = g64 + a.segV;
   float *As32 = reinterpret_cast<float *>(o64 + a.segV);
-  float *g32 = As32 + a.segA;
+  float *g32 = reinterpret_cast<float *>(g64);  // the inner iteration's vectors
   float *o1 = g32 + a.segV;
   float *o2 = o1 + a.segV;
   // in-launch difficulty ordering first: it borrows the start of the warp
   // regions (and ends with a block barrier)
   if (a.ord_ws)
     order_prologue<false>(a, reinterpret_cast<int *>(smem_raw + sched_smem_bytes(nsch)));
-  for (int i = sl; i < a.segV; i += Lc) {
-    g64[i] = 0.0; o64[i] = 0.0; g32[i] = 0.0f; o1[i] = 0.0f; o2[i] = 0.0f;
-  }
   __syncthreads();
   const SchedWord *sch = sch_s;
   const unsigned g64a = smem_addr(g64), o64a = smem_addr(o64), g32a = smem_addr(g32),
@@ -106,6 +102,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
       // ---- FP64 true residual r = b - A x (x = 0 on the first pass)
       double r[E];
       if (pass > 0) {
+        __syncwarp();  // the inner vectors' last reads
 #pragma unroll
         for (int e = 0; e < E; ++e) g64[sl + e * Lc] = xv[e];
         __syncwarp();
@@ -118,10 +115,15 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
       for (int e = 0; e < E; ++e) {
         const int i = sl + e * Lc;
         const double bi = (has && i < n) ? __ldg(a.b + (size_t)c * n + i) : 0.0;
-        r[e] = pass > 0 ? bi - o64[i] : bi;
-        rr[0] = fma(r[e], r[e], rr[0]);
+        r[e] = pass > 0 && i < n ? bi - o64[i] : bi;
       }
-      rr[0] = seg_sum_x<LC>(rr[0], Lc);
+      if (pass > 0) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) rr[0] = fma(r[e], r[e], rr[0]);
+        rr[0] = seg_sum_x<LC>(rr[0], Lc);
+      } else {
+        rr[0] = bb;  // r = b: the same chain and exact sum
+      }
       if (!done) {
         // ||r|| <= tol ||b|| on the bit patterns; the relative residual itself
         // (a square root and a division) is formed once, at the end
@@ -154,6 +156,12 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
       const double sc64 = wide ? 1.0 / rn64 : 0.0;
       float rf[E], rh[E], p[E], d[E];  // rf also holds s = r - alpha v
       float cc[1] = {0.0f};
+      __syncwarp();  // the FP64 product's last reads
+      // pad rows of the product vectors are never written by the products
+      for (int i = n + sl; i < E * Lc; i += Lc) {
+        o1[i] = 0.0f;
+        o2[i] = 0.0f;
+      }
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const float ce = done ? 0.0f : (wide ? d2f_rn(r[e] * sc64) : d2f_rn(r[e]) * rinv32);
@@ -289,16 +297,18 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
   finish_queue(a, true, warps_total, lane);
 }
 
-template <int E>
-__global__ void __launch_bounds__(256, 2) mixed_refine_kernel(const __grid_constant__ MixedArgs a) {
-  // the automatic choice (at most 3 rows per lane on 8, 16 or 32 lanes) runs
-  // code with the lane count fixed at compile time
-  if constexpr (E >= 2 && E <= 3) {
-    if (a.Lc == 32) return mixed_body<E, 32>(a);
-    if (a.Lc == 16) return mixed_body<E, 16>(a);
-    if (a.Lc == 8) return mixed_body<E, 8>(a);
-  }
-  mixed_body<E, 0>(a);
+// FP32 and FP64 issue and shared memory are each about half busy, so resident
+// warps hide the rest: 20 per SM (96 registers), and 24 (80 registers) with up
+// to 3 rows per lane on 32 lanes, where nothing spills and A in FP64 is not
+// read through L1; 16 (128 registers) beyond 5 rows per lane.  16 / 20 / 24 warps: 150 species x 100,000 cells 1,919 /
+// 1,858 / 2,273 us, 80 x 10,000 117 / 112 / 105, 40 x 20,000 (16 lanes) 114 /
+// 113 / 123.
+template <int E, int LC>
+constexpr bool kMixedMany = E <= 3 && LC == 32;
+template <int E, int LC>
+__global__ void __launch_bounds__(kMixedMany<E, LC> || E > 5 ? 256 : 320, kMixedMany<E, LC> ? 3 : 2)
+    mixed_refine_kernel(const __grid_constant__ MixedArgs a) {
+  mixed_body<E, LC>(a);
 }
 
 }  // namespace camp

@@ -26,7 +26,7 @@ CAMP_DECL(8) CAMP_DECL(9) CAMP_DECL(10) CAMP_DECL(11) CAMP_DECL(12)
 CAMP_DECL(13) CAMP_DECL(14) CAMP_DECL(15) CAMP_DECL(16)
 #define CAMP_DECLM(E)                                                        \
   cudaError_t launch_mixed_##E(const MixedArgs &, int, int, size_t, cudaStream_t); \
-  cudaError_t occ_mixed_##E(int, size_t, int *);
+  cudaError_t occ_mixed_##E(int, int, size_t, int *);
 CAMP_DECLM(1) CAMP_DECLM(2) CAMP_DECLM(3) CAMP_DECLM(4) CAMP_DECLM(5)
 CAMP_DECLM(6) CAMP_DECLM(7) CAMP_DECLM(8) CAMP_DECLM(9) CAMP_DECLM(10)
 CAMP_DECLM(11) CAMP_DECLM(12) CAMP_DECLM(13) CAMP_DECLM(14) CAMP_DECLM(15)
@@ -97,9 +97,9 @@ cudaError_t launch_mixed(int E, const MixedArgs &a, int wpb, int grid,
     default: return cudaErrorInvalidValue;
   }
 }
-cudaError_t mixed_occupancy(int E, int wpb, size_t smem, int *blocks) {
+cudaError_t mixed_occupancy(int E, int Lc, int wpb, size_t smem, int *blocks) {
   switch (E) {
-#define C(E) case E: return occ_mixed_##E(wpb, smem, blocks);
+#define C(E) case E: return occ_mixed_##E(Lc, wpb, smem, blocks);
     C(1) C(2) C(3) C(4) C(5) C(6) C(7) C(8) C(9) C(10) C(11) C(12) C(13)
     C(14) C(15) C(16)
 #undef C
@@ -1834,7 +1834,7 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
     while (sm > h->smem_optin && w > 1) sm = mixed_smem(v, Lc, S->L, --w, &segA, &segV, s64 != 0);
     if (sm > h->smem_optin) continue;
     int occ = 0;
-    if ((e = mixed_occupancy(E, w, sm, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
+    if ((e = mixed_occupancy(E, Lc, w, sm, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
     if (occ * w > best_warps) {  // resident warps per SM; a tie keeps the staged FP64 A
       best_warps = occ * w;
       a64 = s64 != 0;
@@ -1865,7 +1865,7 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
     if (rs != CAMP_OK) return rs;
   }
   int occ = 0;
-  if ((e = mixed_occupancy(E, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
+  if ((e = mixed_occupancy(E, Lc, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int need = (a.ngroups + wpb - 1) / wpb;
   const int grid = std::max(1, std::min(need, h->sms * occ));
