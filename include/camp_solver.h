@@ -151,8 +151,9 @@ camp_status camp_solver_set_arrangement(camp_solver_t h, int arrangement,
  *      64th; in between only the (up to 8) rows where it peaked, picked on
  *      the host from the counts of that full read (copied back without
  *      blocking).  Device scratch: 8 bytes per cell plus 4 per row.
- *      Solves on other streams (camp_solver_solve_host's chunks) use index
- *      order; launches whose warp regions cannot lend the ordering 2,576
+ *      Solves on other streams (camp_solver_solve_host's chunks) and launches
+ *      with at most one group per SM sub-partition, which end with their hardest
+ *      cell in any order, use index order; launches whose warp regions cannot lend the ordering 2,576
  *      bytes of shared memory, or whose cooperative launch the GPU refuses
  *      (fewer SMs available than its occupancy query counts), use mode 2.  Under stream capture the
  *      last picked rows are used as they are (allocate first: run one solve

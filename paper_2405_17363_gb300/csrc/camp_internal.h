@@ -317,9 +317,15 @@ struct MixedArgs {
 };
 // Shared-memory bytes per cell of the refinement kernel: FP32 A, FP64 A when
 // staged, and two FP64 vectors, whose space the three FP32 vectors of the
-// inner iteration share; rounded to 16.
-__host__ __device__ inline size_t mixed_cell_bytes(int segA, int segV, bool a64_smem) {
-  return ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)16 * segV + 15) & ~(size_t)15;
+// inner iteration share; rounded to 16 and, with several cells per warp, to Lc
+// four-byte banks modulo the 32 (at least 16 bytes), so that the warp's cells
+// gather from different banks (24 species, 8 lanes: a multiple of 128 bytes
+// put all four cells of a warp on the same ones).
+__host__ __device__ inline size_t mixed_cell_bytes(int segA, int segV, bool a64_smem, int Lc) {
+  const size_t need = ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)16 * segV + 15) & ~(size_t)15;
+  if (Lc >= 32) return need;
+  const size_t want = Lc < 4 ? 16 : 4 * (size_t)Lc;
+  return need + (want + 128 - need % 128) % 128;
 }
 // a cooperative launch when a.ord_ws is set (grid at most SMs x occupancy)
 cudaError_t launch_mixed(int E, const MixedArgs &a, int warps_per_block,

@@ -31,7 +31,7 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
   const int seg = LC ? lane / LC : lane >> a.log2Lc;
   const int sl = lane & (Lc - 1);
   const int n = a.n, nnz = a.nnz;
-  const size_t cellBytes = mixed_cell_bytes(a.segA, a.segV, a.a64_smem);
+  const size_t cellBytes = mixed_cell_bytes(a.segA, a.segV, a.a64_smem, Lc);
   unsigned char *wb = smem_raw + sched_smem_bytes(nsch) +
                       ((size_t)warp * a.k + seg) * cellBytes;
   double *As = reinterpret_cast<double *>(wb);

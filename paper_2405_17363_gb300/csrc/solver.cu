@@ -658,7 +658,7 @@ size_t mixed_smem(const View &v, int Lc, int L, int wpb, int *segA, int *segV, b
   *segA = (L * Lc + 1) & ~1;  // A in slot order
   *segV = (E * Lc + 1) & ~1;
   const size_t sch = sched_smem_bytes(L * Lc);
-  return sch + (size_t)wpb * k * mixed_cell_bytes(*segA, *segV, a64_smem);
+  return sch + (size_t)wpb * k * mixed_cell_bytes(*segA, *segV, a64_smem, Lc);
 }
 
 // Automatic arrangement: the most cells per warp (fewest lanes per cell) that
@@ -799,6 +799,13 @@ camp_status ensure_order_capacity(camp_solver_t h, int cells, cudaStream_t st) {
   return CAMP_OK;
 }
 
+// Whether ordering the cells can shorten a launch: with at most one group per
+// SM sub-partition every group starts at once on an FP64 unit of its own, and
+// the launch ends with its hardest cell whatever the order, so the prologue
+// (and the cooperative launch) would only delay it (64 cells of 30 species: 36
+// us with it, 28 without; 600 cells of 80 species: 45 and 37).
+bool worth_ordering(camp_solver_t h, int ngroups) { return ngroups > 4 * h->sms; }
+
 // In-launch ordering of the fused-assembly and Newton launches (orderings 1
 // and 2): cells classified by gamma, as the plain launch classifies them by
 // its sampled diagonal (there is no matrix before a cell is assembled).
@@ -806,7 +813,7 @@ camp_status ensure_order_capacity(camp_solver_t h, int cells, cudaStream_t st) {
 // shared memory.
 camp_status setup_gamma_ordering(camp_solver_t h, WarpArgs &a, size_t smem_free,
                                  cudaStream_t st) {
-  if (!h->ordering || a.cells <= 1 || smem_free < kOrdSmemBytes) return CAMP_OK;
+  if (!h->ordering || !worth_ordering(h, a.ngroups) || smem_free < kOrdSmemBytes) return CAMP_OK;
   camp_status rs = ensure_order_capacity(h, a.cells, st);
   if (rs != CAMP_OK) return rs;
   cudaError_t e;
@@ -846,7 +853,7 @@ camp_status setup_ordering(camp_solver_t h, Args &a, const double *A_vals, size_
                            cudaStream_t st, bool *calibrate) {
   const int cells = a.cells;
   *calibrate = false;
-  if (!h->ordering || cells <= 1) return CAMP_OK;
+  if (!h->ordering || !worth_ordering(h, a.ngroups)) return CAMP_OK;
   cudaError_t e = cudaSuccess;
   const bool inl = h->ordering == 1 && smem_free >= kOrdSmemBytes;
   if (inl) {
