@@ -38,6 +38,36 @@ __host__ __device__ inline size_t sched_smem_bytes(int nsch) {
   return (((size_t)nsch * sizeof(SchedWord)) + 15) & ~(size_t)15;
 }
 
+// Tables of a mass-action mechanism for one lane count, read through L1.  A
+// cell's chains (the Jacobian terms of a matrix entry, the rate terms of a row)
+// may be summed by any lane, each in its order: they are sorted by length and
+// taken in groups of Lc, one per lane, all lanes running as many steps as the
+// group's longest (shorter chains start with steps that add zero), so the
+// loops are uniform and the lanes balanced.  Offsets are bytes from the cell's
+// matrix block; the two entries after it hold 1.0 and 0.0 while the tables
+// are used, the third takes what idle lanes store.
+struct MechTables {
+  // Jacobian: runs of groups {steps, groups}; per group and lane {start value
+  // of the chain (its leading constant terms summed on the host, in order),
+  // place of the entry, high word of its identity part}; per step and lane
+  // {coefficient, offset of its concentration or of 1.0}
+  const int2 *jrun;
+  const int4 *jhead, *jstep;
+  int jruns;
+  // rates f(y), in chunks of at most the matrix block's doubles: per chunk
+  // {rounds of second-order reactions, rounds of first-order ones, runs of
+  // row groups, 0}; per round and lane {rate constant, offsets of y_a | y_b
+  // << 16 in units of 8 bytes, offset of the reaction's rate}; per group and
+  // lane the row's offset in the rate vector's buffer; per step and lane the
+  // reaction's rate offset | sign << 31
+  const int4 *rchunk;
+  int rchunks;
+  const int4 *rate;
+  const int2 *rrun;
+  const int *rhead;
+  const unsigned *rstep;
+};
+
 // Arguments of the warp-packed kernel: Lc lanes per cell, k = 32/Lc cells per
 // warp ("segments"), E rows per lane (template), one group of k consecutive
 // cells per warp at a time.
@@ -117,24 +147,15 @@ struct WarpArgs {
   unsigned *ord_hits;
   int *ord_err;
   long long ord_wait;
-  // Fused assembly (assemble_bicgstab_kernel only): the cell's matrix is
-  // built in shared memory as A = I - gamma J(conc) instead of read from A.
-  // Lane sl runs tcount terms p: J[place tmeta >> 11] +=
-  // tval * (conc[(tmeta & 0x7ff) - 1] or 1 when that field is 0); arrays
-  // are laid out [p][lane], padding terms add zero.
+  // Fused assembly (assemble_bicgstab_kernel and newton_bicgstab_kernel): the
+  // cell's matrix is built in shared memory as A = I - gamma J(conc) instead of
+  // read from A; mechanism tables, see MechTables.
   const double *conc;      // [cells x n]
   const double *gamma;     // [cells]
-  const double *tval;      // [tcount x Lc] sign * rate constant
-  const int *tmeta;        // [tcount x Lc] species + 1 | place (pair_pos) << 11
-  int tcount;
-  // Newton corrector (newton_bicgstab_kernel only): lane sl accumulates
-  // f[row sl + e*Lc] += rval * y[a] * (y[b] or 1) over its rcount terms,
-  // rmeta = (a + 1) | (b + 1) << 11 | e << 22 ([p][lane]); the history term
-  // is read from b, y (in: initial guess, out: solution) from x, the linear
-  // tolerance and iteration cap from tol and maxit.
-  const double *rval;
-  const int *rmeta;
-  int rcount;
+  // Newton corrector (newton_bicgstab_kernel only): the history term is read
+  // from b, y (in: initial guess, out: solution) from x, the linear tolerance
+  // and iteration cap from tol and maxit.
+  MechTables mech;
   double newton_tol;
   int max_newton;
   int *newton_iters;       // [cells]

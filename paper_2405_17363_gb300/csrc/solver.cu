@@ -327,6 +327,7 @@ Schedule build_schedule(int n, const std::vector<int> &rp,
 struct Slots {
   int Lc = 0, L = 0, npads = 0;
   std::vector<int> dst;      // [nnz] slot (j * Lc + lane) of each A entry
+  std::vector<int> dentry;   // [n] A entry of each row's diagonal
   unsigned ends[kEndWords] = {};
   SchedWord *d_words = nullptr;
   int *d_src = nullptr;      // word_pos places
@@ -375,28 +376,25 @@ cudaError_t upload(T **dst, const std::vector<T> &src) {
 
 // Mass-action mechanism attached to a handle for the fused assembly: its
 // Jacobian terms in reaction order (pattern entry, concentration factor,
-// signed rate constant) and, per lanes-per-cell choice, the terms grouped by
-// schedule slot on the device.
+// signed rate constant), its reactions and the rate terms of every row, and,
+// per lanes-per-cell choice, their tables on the device.
 struct MechTerms {
-  int count = 0;               // Jacobian terms per lane (padded)
-  int *d_tmeta = nullptr;
-  double *d_tval = nullptr;
-  int rcount = 0;              // rate terms per lane (padded)
-  int *d_rmeta = nullptr;
-  double *d_rval = nullptr;
+  MechTables t = {};
   void release() {
-    cudaFree(d_tmeta);
-    cudaFree(d_tval);
-    cudaFree(d_rmeta);
-    cudaFree(d_rval);
+    for (const void *p : {(const void *)t.jrun, (const void *)t.jhead, (const void *)t.jstep,
+                          (const void *)t.rchunk, (const void *)t.rate, (const void *)t.rrun,
+                          (const void *)t.rhead, (const void *)t.rstep})
+      cudaFree(const_cast<void *>(p));
   }
 };
 struct Mechanism {
   int R = 0;
   std::vector<int> entry, spec;  // Jacobian terms: CSR entry, factor species
   std::vector<double> val;
-  std::vector<int> rrow, ra, rb;  // rate terms: row of f, factor species
-  std::vector<double> rk;         // signed rate constant
+  std::vector<int> ra, rb;     // reactions: factor species (rb -1: first order)
+  std::vector<double> rk;      // rate constants
+  std::vector<int> rrow, rrx;  // rate terms in reaction order: row of f, reaction
+  std::vector<char> rneg;      // consumed (the rate enters with a minus sign)
   std::map<int, MechTerms> by_lanes;
 };
 
@@ -464,6 +462,7 @@ cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<uns
                          const std::vector<int> &src, const std::vector<int> &dentry) {
   S.Lc = Lc;
   S.L = L;
+  S.dentry = dentry;
   S.dst.assign(nnz, -1);
   std::vector<SchedWord> words((size_t)L * Lc);
   sched::pack_words(L, Lc, word.data(), words.data());
@@ -1598,14 +1597,15 @@ camp_status camp_solver_set_mechanism(camp_solver_t h, int R,
     }
     // rate terms of f: the reaction's rate leaves a (and b), enters c
     const int rows[3] = {a, b, c};
-    const double sg[3] = {-k, -k, k};
     for (int q = 0; q < 3; ++q) {
       if (rows[q] < 0) continue;
       M.rrow.push_back(rows[q]);
-      M.ra.push_back(a);
-      M.rb.push_back(b);
-      M.rk.push_back(sg[q]);
+      M.rrx.push_back(r);
+      M.rneg.push_back(q < 2);
     }
+    M.ra.push_back(a);
+    M.rb.push_back(b);
+    M.rk.push_back(k);
   }
   for (auto &kv : h->mech.by_lanes) kv.second.release();
   h->mech = std::move(M);
@@ -1615,53 +1615,149 @@ camp_status camp_solver_set_mechanism(camp_solver_t h, int R,
 namespace camp {
 namespace {
 
-// Per-lane term lists of the handle's mechanism for Lc lanes per cell, padded
-// to the longest lane and laid out [term][lane]: the Jacobian terms of the
-// lane's slots (tmeta = (species + 1) | place << 11) and the rate terms of
-// the lane's rows (rmeta = (a + 1) | (b + 1) << 11 | e << 22, row sl + e Lc).
-cudaError_t mech_terms(Mechanism &mech, int Lc, const Slots &S, MechTerms **out) {
+// Chains (by id) sorted by length, longest first, in groups of Lc; runs of
+// groups of the same step count.
+struct ChainGroups {
+  std::vector<int> order;  // ids; group g's lane q takes order[g * Lc + q]
+  std::vector<int2> runs;  // {steps, groups}
+};
+ChainGroups group_chains(const std::vector<int> &len, int Lc) {
+  ChainGroups G;
+  G.order.resize(len.size());
+  std::iota(G.order.begin(), G.order.end(), 0);
+  std::stable_sort(G.order.begin(), G.order.end(), [&](int p, int q) { return len[p] > len[q]; });
+  for (size_t i = 0; i < G.order.size(); i += Lc) {
+    const int steps = len[G.order[i]];
+    if (G.runs.empty() || G.runs.back().x != steps) G.runs.push_back(make_int2(steps, 0));
+    ++G.runs.back().y;
+  }
+  return G;
+}
+
+int4 with_double(double v, int z, int w) {
+  unsigned long long u;
+  memcpy(&u, &v, sizeof u);
+  return make_int4((int)(unsigned)u, (int)(unsigned)(u >> 32), z, w);
+}
+
+// The device tables (MechTables) of the handle's mechanism for Lc lanes per
+// cell on the slots S.
+cudaError_t mech_terms(Mechanism &mech, int n, int Lc, const Slots &S, MechTerms **out) {
   auto it = mech.by_lanes.find(Lc);
   if (it != mech.by_lanes.end()) {
     *out = &it->second;
     return cudaSuccess;
   }
-  auto pad = [Lc](std::vector<std::vector<std::pair<double, int>>> &lane,
-                  std::vector<double> &val, std::vector<int> &meta, auto idle) {
-    size_t M = 1;
-    for (auto &l : lane) M = std::max(M, l.size());
-    val.assign(M * Lc, 0.0);
-    meta.assign(M * Lc, 0);
-    for (size_t p = 0; p < M; ++p)
-      for (int q = 0; q < Lc; ++q) meta[p * Lc + q] = idle(q);
-    for (int q = 0; q < Lc; ++q)
-      for (size_t p = 0; p < lane[q].size(); ++p) {
-        val[p * Lc + q] = lane[q][p].first;
-        meta[p * Lc + q] = lane[q][p].second;
+  const int E = (n + Lc - 1) / Lc;
+  const int segA = (S.L * Lc + 1) & ~1, segV = ((E * Lc + 1) + 1) & ~1;
+  const int one = segA, zero = segA + 1, idle = segA + 2;  // doubles from the matrix block
+  auto conc = [&](int sp) { return sp < 0 ? one : segA + 2 * segV + sp; };
+  const int nnz = (int)S.dst.size();
+  // Jacobian: the terms of every entry in reaction order; a chain's leading
+  // constant terms are summed here, as the chain would (fma(v, 1, acc))
+  std::vector<std::vector<int>> terms(nnz);
+  for (size_t q = 0; q < mech.entry.size(); ++q) terms[mech.entry[q]].push_back((int)q);
+  std::vector<double> start(nnz, 0.0);
+  std::vector<int> lead(nnz, 0), len(nnz, 0);
+  for (int k = 0; k < nnz; ++k) {
+    while (lead[k] < (int)terms[k].size() && mech.spec[terms[k][lead[k]]] < 0)
+      start[k] += mech.val[terms[k][lead[k]++]];
+    len[k] = (int)terms[k].size() - lead[k];
+  }
+  const ChainGroups J = group_chains(len, Lc);
+  std::vector<char> diag(nnz, 0);
+  for (int k : S.dentry) diag[k] = 1;
+  std::vector<int4> jhead, jstep;
+  size_t i0 = 0;
+  for (const int2 &run : J.runs)
+    for (int g = 0; g < run.y; ++g, i0 += Lc) {
+      for (int q = 0; q < Lc; ++q) {
+        if (i0 + q >= J.order.size()) {
+          jhead.push_back(with_double(0.0, 8 * idle, 0));
+          continue;
+        }
+        const int k = J.order[i0 + q], t = S.dst[k];
+        jhead.push_back(with_double(start[k], 8 * pair_pos(t / Lc, t % Lc, S.L, Lc),
+                                    diag[k] ? 0x3ff00000 : 0));
       }
-    return (int)M;
-  };
-  std::vector<std::vector<std::pair<double, int>>> lane(Lc), rlane(Lc);
-  for (size_t q = 0; q < mech.entry.size(); ++q) {
-    const int t = S.dst[mech.entry[q]];
-    lane[t % Lc].push_back(
-        {mech.val[q], (mech.spec[q] + 1) | (pair_pos(t / Lc, t % Lc, S.L, Lc) << 11)});
+      for (int s = 0; s < run.x; ++s)
+        for (int q = 0; q < Lc; ++q) {
+          const int k = i0 + q < J.order.size() ? J.order[i0 + q] : -1;
+          const int u = k < 0 ? -1 : s - (run.x - len[k]);
+          if (u < 0) {
+            jstep.push_back(with_double(0.0, 8 * one, 0));
+            continue;
+          }
+          const int z = terms[k][lead[k] + u];
+          jstep.push_back(with_double(mech.val[z], 8 * conc(mech.spec[z]), 0));
+        }
+    }
+  // rates: chunks of reactions whose rates fit the matrix block
+  std::vector<int4> rchunk, rate;
+  std::vector<int2> rrun;
+  std::vector<int> rhead;
+  std::vector<unsigned> rstep;
+  size_t z0 = 0;
+  for (int r0 = 0; r0 < mech.R; r0 += segA) {
+    const int r1 = std::min(mech.R, r0 + segA);
+    int rounds[2] = {0, 0};
+    for (int order = 0; order < 2; ++order) {  // second order, then first
+      std::vector<int> rx;
+      for (int r = r0; r < r1; ++r)
+        if ((mech.rb[r] < 0) == (order == 1)) rx.push_back(r);
+      rounds[order] = ((int)rx.size() + Lc - 1) / Lc;
+      for (int i = 0; i < rounds[order] * Lc; ++i) {
+        if (i >= (int)rx.size()) {
+          rate.push_back(with_double(0.0, (int)((unsigned)one | (unsigned)one << 16), 8 * idle));
+          continue;
+        }
+        const int r = rx[i];
+        rate.push_back(with_double(mech.rk[r],
+                                   (int)((unsigned)conc(mech.ra[r]) |
+                                         (unsigned)conc(mech.rb[r]) << 16),
+                                   8 * (r - r0)));
+      }
+    }
+    std::vector<std::vector<unsigned>> row(n);
+    for (; z0 < mech.rrow.size() && mech.rrx[z0] < r1; ++z0)
+      row[mech.rrow[z0]].push_back((unsigned)(8 * (mech.rrx[z0] - r0)) |
+                                   (mech.rneg[z0] ? 0x80000000u : 0u));
+    std::vector<int> rlen(n);
+    for (int i = 0; i < n; ++i) rlen[i] = (int)row[i].size();
+    ChainGroups G = group_chains(rlen, Lc);
+    size_t g0 = 0;
+    int runs = 0;
+    for (const int2 &run : G.runs) {
+      if (run.x == 0) break;  // rows without a term
+      rrun.push_back(run);
+      ++runs;
+      for (int g = 0; g < run.y; ++g, g0 += Lc) {
+        for (int q = 0; q < Lc; ++q)
+          rhead.push_back(8 * (g0 + q < G.order.size() ? G.order[g0 + q] : n));
+        for (int s = 0; s < run.x; ++s)
+          for (int q = 0; q < Lc; ++q) {
+            const int i = g0 + q < G.order.size() ? G.order[g0 + q] : -1;
+            const int u = i < 0 ? -1 : s - (run.x - rlen[i]);
+            rstep.push_back(u < 0 ? (unsigned)(8 * zero) : row[i][u]);
+          }
+      }
+    }
+    rchunk.push_back(make_int4(rounds[0], rounds[1], runs, 0));
   }
-  for (size_t q = 0; q < mech.rrow.size(); ++q) {
-    const int row = mech.rrow[q];
-    rlane[row % Lc].push_back(
-        {mech.rk[q], (mech.ra[q] + 1) | ((mech.rb[q] + 1) << 11) | ((row / Lc) << 22)});
-  }
-  std::vector<double> tval, rval;
-  std::vector<int> tmeta, rmeta;
   MechTerms T;
-  // a padding term adds zero to a place (a row) of its own lane
-  T.count = pad(lane, tval, tmeta, [&](int q) { return pair_pos(0, q, S.L, Lc) << 11; });
-  T.rcount = pad(rlane, rval, rmeta, [](int) { return 0; });
+  T.t.jruns = (int)J.runs.size();
+  T.t.rchunks = (int)rchunk.size();
+  auto put = [](auto &dst, const auto &src) {
+    auto *p = const_cast<std::remove_const_t<std::remove_pointer_t<std::decay_t<decltype(dst)>>> *>(dst);
+    const cudaError_t e = upload(&p, src);
+    dst = p;
+    return e;
+  };
   cudaError_t e;
-  if ((e = upload(&T.d_tval, tval)) != cudaSuccess ||
-      (e = upload(&T.d_tmeta, tmeta)) != cudaSuccess ||
-      (e = upload(&T.d_rval, rval)) != cudaSuccess ||
-      (e = upload(&T.d_rmeta, rmeta)) != cudaSuccess) {
+  if ((e = put(T.t.jrun, J.runs)) != cudaSuccess || (e = put(T.t.jhead, jhead)) != cudaSuccess ||
+      (e = put(T.t.jstep, jstep)) != cudaSuccess || (e = put(T.t.rchunk, rchunk)) != cudaSuccess ||
+      (e = put(T.t.rate, rate)) != cudaSuccess || (e = put(T.t.rrun, rrun)) != cudaSuccess ||
+      (e = put(T.t.rhead, rhead)) != cudaSuccess || (e = put(T.t.rstep, rstep)) != cudaSuccess) {
     T.release();
     return e;
   }
@@ -1689,7 +1785,7 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
     return cuda_fail(e, "schedule upload");
   if (S->L > 2047) return fail(CAMP_EUNSUPPORTED, "more than 2047 slots per lane");
   MechTerms *T = nullptr;
-  if ((e = mech_terms(h->mech, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
+  if ((e = mech_terms(h->mech, v.n, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
   int wpb = h->wpb > 0 ? h->wpb : 4;
   int segA = 0, segV = 0, segStride = 0;
   size_t smem = warp_smem(v, Lc, S->L, wpb, &segA, &segV, &segStride, extra_vectors);
@@ -1710,8 +1806,7 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
   a.dslot = S->d_dslot;
   a.x0_given = 0;
   a.queue = h->d_queue;
-  a.tval = T->d_tval; a.tmeta = T->d_tmeta; a.tcount = T->count;
-  a.rval = T->d_rval; a.rmeta = T->d_rmeta; a.rcount = T->rcount;
+  a.mech = T->t;
   *pa = a;
   *pE = E;
   *pwpb = wpb;

@@ -82,6 +82,9 @@ __device__ __forceinline__ void lds(double &v, unsigned a) {
 __device__ __forceinline__ void lds(float &v, unsigned a) {
   asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
 }
+__device__ __forceinline__ void sts(unsigned a, double v) {
+  asm volatile("st.shared.f64 [%0], %1;" :: "r"(a), "d"(v) : "memory");
+}
 // *a = v when flag != 0, as one predicated store (no branch)
 __device__ __forceinline__ void sts_if(unsigned flag, unsigned a, double v) {
   asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q st.shared.f64 [%1], %2;\n\t}"

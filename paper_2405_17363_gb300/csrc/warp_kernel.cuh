@@ -80,6 +80,92 @@ struct LaneRows<E, false> {
   __device__ __forceinline__ double &operator[](int e) { return p[e * Lc]; }
 };
 
+// The constants of the mechanism tables, in the first entries of the gathered
+// vector (MechTables).
+__device__ __forceinline__ void table_constants(const WarpArgs &a, double *Abase, int sl) {
+  if (sl == 0) {
+    Abase[a.segA] = 1.0;
+    Abase[a.segA + 1] = 0.0;
+  }
+}
+
+// A = I - gamma J(conc), every entry by the chain of multiply-adds of its
+// terms and one for the identity part (ab: shared address of the matrix
+// block).  FP64-bound: 42 + 36 multiply-adds per lane at 80 species, 200
+// reactions, 16 lanes, against 65 + 36 with every lane summing the terms of its
+// own slots in shared memory.
+__device__ __forceinline__ void assemble_matrix(const MechTables &m, unsigned ab, double gam,
+                                                int sl, int Lc) {
+  const int4 *head = m.jhead + sl, *step = m.jstep + sl;
+  for (int r = 0; r < m.jruns; ++r) {
+    const int2 run = __ldg(m.jrun + r);
+#pragma unroll 2
+    for (int g = 0; g < run.y; ++g) {
+      const int4 h = __ldg(head);
+      head += Lc;
+      double acc = __hiloint2double(h.y, h.x);
+#pragma unroll 2
+      for (int t = 0; t < run.x; ++t) {
+        const int4 w = __ldg(step);
+        step += Lc;
+        double y;
+        lds(y, ab + (unsigned)w.z);
+        acc = fma(__hiloint2double(w.y, w.x), y, acc);
+      }
+      sts(ab + (unsigned)h.z, fma(-gam, acc, __hiloint2double(h.w, 0)));
+    }
+  }
+}
+
+// f(y) += the mass-action rates at the concentrations in shared memory (fb:
+// shared address of f): each reaction's rate once, into the matrix block's
+// space, then every row's sum of them in reaction order.
+__device__ __forceinline__ void mass_action_rates(const MechTables &m, unsigned ab, unsigned fb,
+                                                  int sl, int Lc) {
+  const int4 *rate = m.rate + sl;
+  const int2 *rrun = m.rrun;
+  const int *rhead = m.rhead + sl;
+  const unsigned *rstep = m.rstep + sl;
+  for (int c = 0; c < m.rchunks; ++c) {
+    const int4 chunk = __ldg(m.rchunk + c);
+#pragma unroll 2
+    for (int q = 0; q < chunk.x + chunk.y; ++q) {
+      const int4 w = __ldg(rate);
+      rate += Lc;
+      double ya, v;
+      lds(ya, ab + 8u * ((unsigned)w.z & 0xffffu));
+      v = __dmul_rn(__hiloint2double(w.y, w.x), ya);
+      if (q < chunk.x) {
+        double yb;
+        lds(yb, ab + 8u * ((unsigned)w.z >> 16));
+        v = __dmul_rn(v, yb);
+      }
+      sts(ab + (unsigned)w.w, v);
+    }
+    __syncwarp();
+    for (int r = 0; r < chunk.z; ++r) {
+      const int2 run = __ldg(rrun++);
+      for (int g = 0; g < run.y; ++g) {
+        const unsigned f = fb + (unsigned)__ldg(rhead);
+        rhead += Lc;
+        double acc;
+        lds(acc, f);
+#pragma unroll 2
+        for (int t = 0; t < run.x; ++t) {
+          const unsigned w = __ldg(rstep);
+          rstep += Lc;
+          double v;
+          lds(v, ab + (w & 0x7fffffffu));
+          acc = __dadd_rn(acc, __hiloint2double(__double2hiint(v) ^ (int)(w & 0x80000000u),
+                                                __double2loint(v)));
+        }
+        sts(f, acc);
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // Newton corrector of the implicit step G(y) = y - gamma f(y) - a = 0 for
 // the segment's cell (a: history term in b; y: initial guess in x, replaced
 // by the solution): each iteration evaluates the mass-action rates f(y),
@@ -92,7 +178,7 @@ struct LaneRows<E, false> {
 // after the update, so no register holds it across the linear solve.
 template <int E, class Solve>
 __device__ __forceinline__ void newton_loop(const WarpArgs &a, bool has, bool &live, int c,
-                                            int sl, int Lc, int n, double *o1, double *o2,
+                                            int sl, int Lc, int n, double *Abase, double *o1, double *o2,
                                             double *nrh, double (&xv)[E], int &st, int &it,
                                             double &resid, Solve &stage_and_solve) {
   double *yc = a.x + (size_t)c * n;  // the iterate (c is in range whenever has)
@@ -103,25 +189,16 @@ __device__ __forceinline__ void newton_loop(const WarpArgs &a, bool has, bool &l
   double upd = 0.0, lres = 0.0;
   bool act = has && any;
   while (__any_sync(kFull, act)) {
-    // the iterate to the concentration buffer, f(y) accumulated in o1 (each
-    // lane adds the terms of its own rows)
+    // the iterate to the concentration buffer, f(y) to o1
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int i = sl + e * Lc;
       o2[i] = (has && i < n) ? yc[i] : 0.0;
       o1[i] = 0.0;
     }
+    table_constants(a, Abase, sl);
     __syncwarp();
-    const double *rv = a.rval + sl;
-    const int *rm = a.rmeta + sl;
-    for (int q = 0; q < a.rcount; ++q) {
-      const int meta = __ldg(rm + q * Lc);
-      const int ya = (meta & 0x7ff) - 1, yb = ((meta >> 11) & 0x7ff) - 1;
-      const int row = sl + ((meta >> 22) & 0xff) * Lc;
-      double term = __ldg(rv + q * Lc) * (ya >= 0 ? o2[ya] : 1.0);
-      if (yb >= 0) term *= o2[yb];
-      o1[row] += term;
-    }
+    mass_action_rates(a.mech, smem_addr(Abase), smem_addr(o1), sl, Lc);
     // right-hand side -G(y) = a - (y - gamma f(y))
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -237,29 +314,15 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   // ---- stage the cell's matrix values in slot order (Sec. 3.1: one cell,
   // one team); the transposed view's permutation is folded into src
   if (SRC == kSrcAssembled || SRC == kSrcNewton) {
-    // J accumulates in place in the lane's own slots, then A = I - gamma J
-    for (int j = 0; j < a.L; ++j) Abase[pair_pos(j, sl, a.L, Lc)] = 0.0;
     // the cell's concentrations go to the (not yet used) t-product buffer
     // (the Newton launch has put the current iterate there)
     if (SRC == kSrcAssembled && live)
       for (int i = sl; i < n; i += Lc) o2[i] = __ldg(a.conc + (size_t)c * n + i);
+    table_constants(a, Abase, sl);
     __syncwarp();
     const double gam = live ? __ldg(a.gamma + c) : 0.0;
-    const double *tv = a.tval + sl;
-    const int *tm = a.tmeta + sl;
-    for (int p = 0; p < a.tcount; ++p) {
-      const int meta = __ldg(tm + p * Lc);
-      const int sp = (meta & 0x7ff) - 1;
-      double *dst = Abase + (meta >> 11);
-      *dst = fma(__ldg(tv + p * Lc), sp >= 0 ? o2[sp] : 1.0, *dst);
-    }
-    for (int j = 0; j < a.L; ++j) {
-      const SchedWord w = sch[word_pos(j, sl, a.L, Lc)];  // this lane's word for slot j
-      const bool dg = __ldg(a.src + word_pos(j, sl, a.L, Lc)) >= 0 &&
-                      (w & kSlotRowMask) == (w >> 16);
-      double *t = Abase + pair_pos(j, sl, a.L, Lc);
-      *t = fma(-gam, *t, dg ? 1.0 : 0.0);
-    }
+    zero_padding(Abase, a.pads, a.npads, a.L, sl, Lc);
+    assemble_matrix(a.mech, smem_addr(Abase), gam, sl, Lc);
   } else if (ASMEM) {
     // coalesced read of the cell's A row, scattered into slot order; each lane
     // zeroes its own padding slots (never a scatter target)
@@ -502,7 +565,7 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   };  // stage_and_solve
 
   if (SRC == kSrcNewton) {
-    newton_loop<E>(a, has, live, c, sl, Lc, n, o1, o2, nrh, xv, st, it, resid,
+    newton_loop<E>(a, has, live, c, sl, Lc, n, Abase, o1, o2, nrh, xv, st, it, resid,
                    stage_and_solve);
     return;
   }
