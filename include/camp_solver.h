@@ -317,7 +317,7 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
  * of every cell is that of camp_solver_solve with the automatic arrangement.
  * The SpMV schedule and the diagonal positions, which a handle keeps in
  * device memory of its own, are staged instead into one static device array
- * of 256 KiB inside the library, which every GPU that loads the library holds
+ * of 256 KiB (and as much again for a second copy of the entry map) inside the library, which every GPU that loads the library holds
  * until the process exits; a pattern whose schedule and diagonal positions do
  * not fit returns CAMP_EUNSUPPORTED before any work is enqueued, as does
  * n > 512.  No cudaMalloc, cudaFree or other allocating routine is called.

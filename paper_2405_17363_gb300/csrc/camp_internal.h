@@ -19,6 +19,9 @@ namespace camp {
 typedef unsigned int SchedWord;
 constexpr unsigned kSlotEnd = 1u, kSlotRowMask = 0xfffcu;
 constexpr int kSlotBlock = 4;  // slots per word block
+// A dst map's second copy starts here: at an odd int, so that its entry 1 is
+// 8-byte aligned (the map has dst_odd(nnz) + nnz ints).
+__host__ __device__ inline int dst_odd(int nnz) { return nnz | 1; }
 // Words of a launch's row-end mask, one bit per slot; slots past it are taken
 // as row ends of some lane (what every slot of so long a product is anyway).
 constexpr int kEndWords = 8;
@@ -85,7 +88,7 @@ struct WarpArgs {
   int *status;             // [cells] or null
   const SchedWord *sched;  // [L x Lc] slot words (word_pos)
   const int *src;          // [L x Lc] A entry of each slot (word_pos; transposed view: permuted), -1 pad
-  const int *dst;          // [nnz] place (pair_pos) of each A entry (pattern order)
+  const int *dst;          // [nnz] place (pair_pos) of each A entry (pattern order), twice (dst_odd)
   const int *pads;         // [npads] places (pair_pos) of the padding slots; npads < 0: [Lc] each
   int npads;               // lane's first padding slot (all its later ones are padding too)
   unsigned ends[kEndWords];  // bit j: some lane ends a row in slot j

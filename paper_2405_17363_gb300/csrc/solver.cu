@@ -490,10 +490,15 @@ cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<uns
   }
   cudaError_t e = upload(&S.d_words, words);
   if (e == cudaSuccess) e = upload(&S.d_src, psrc);
-  if (e == cudaSuccess) e = upload(&S.d_dst, dst);
+  auto twice = [nnz](std::vector<int> v) {
+    v.resize((size_t)dst_odd(nnz) + nnz);
+    std::copy(v.begin(), v.begin() + nnz, v.begin() + dst_odd(nnz));
+    return v;
+  };
+  if (e == cudaSuccess) e = upload(&S.d_dst, twice(dst));
   if (e == cudaSuccess) e = upload(&S.d_dslot, dslot);
   if (e == cudaSuccess) e = upload(&S.d_pads, pads);
-  if (e == cudaSuccess) e = upload(&S.d_dst32, dst32);
+  if (e == cudaSuccess) e = upload(&S.d_dst32, twice(dst32));
   if (e == cudaSuccess) e = upload(&S.d_dslot32, dslot32);
   if (e == cudaSuccess) e = upload(&S.d_pads32, pads32);
   if (e == cudaSuccess) e = upload(&S.d_dentry, dentry);
@@ -2300,11 +2305,14 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
 namespace camp {
 namespace {
 constexpr size_t kNoAllocScratchBytes = 256 * 1024;
+// the second copy of the entry map (dst_odd), beside what the limit counts
+constexpr size_t kNoAllocMapBytes = 65536 * sizeof(int) + 64;
 constexpr int kNoAllocMaxDevices = 64;
 }  // namespace
 }  // namespace camp
 
-static __device__ __align__(256) unsigned char g_noalloc_scratch[camp::kNoAllocScratchBytes];
+static __device__ __align__(256) unsigned char
+    g_noalloc_scratch[camp::kNoAllocScratchBytes + camp::kNoAllocMapBytes];
 
 namespace camp {
 namespace {
@@ -2313,7 +2321,7 @@ std::mutex g_noalloc_mu;                              // guards the host buffers
 void *g_noalloc_dev[kNoAllocMaxDevices];              // device address of the scratch
 unsigned g_noalloc_words[kNoAllocScratchBytes / sizeof(unsigned)];      // host form
 SchedWord g_noalloc_packed[kNoAllocScratchBytes / sizeof(SchedWord)];  // device form
-int g_noalloc_dst[kNoAllocScratchBytes / sizeof(int)];
+int g_noalloc_dst[2 * 65536 + 16];
 int g_noalloc_padfrom[32];
 unsigned g_noalloc_ends[kEndWords];
 int g_noalloc_entry[kNoAllocScratchBytes / sizeof(SchedWord)];
@@ -2339,7 +2347,7 @@ int noalloc_schedule(int n, const int *rp, const int *ci, int Lc, size_t cap_slo
   for (int j = 0; j < L; ++j)
     for (int q = 0; q < Lc; ++q) {
       const int k = g_noalloc_entry[(size_t)j * Lc + q];
-      if (k >= 0) g_noalloc_dst[k] = pair_pos(j, q, L, Lc);
+      if (k >= 0) g_noalloc_dst[k] = g_noalloc_dst[dst_odd(rp[n]) + k] = pair_pos(j, q, L, Lc);
     }
   for (int r = 0; r < n; ++r)
     g_noalloc_dslot[r] = pair_pos(g_noalloc_dslot[r] / Lc, g_noalloc_dslot[r] % Lc, L, Lc);
@@ -2389,8 +2397,8 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
     if (g_noalloc_diag[i] < 0) return fail(CAMP_EPATTERN, "diagonal entry missing in row %d", i);
   }
   // scratch layout, 16-byte aligned pieces: [diagonal slots, n ints]
-  // [first padding slot per lane, 32 ints][slot of every entry, nnz ints]
-  // [slot words, L*Lc]
+  // [first padding slot per lane, 32 ints][slot words, L*Lc][place of every
+  // entry, nnz ints, twice]; the limit counts the places once
   const size_t diag_bytes = ((size_t)n * sizeof(int) + 15) & ~(size_t)15;
   const size_t pad_bytes = 32 * sizeof(int);
   const size_t dst_bytes = ((size_t)nnz * sizeof(int) + 15) & ~(size_t)15;
@@ -2442,8 +2450,10 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
   a.pads = (const int *)(scratch + diag_bytes);
   a.npads = -1;  // per lane: the first padding slot
   memcpy(a.ends, g_noalloc_ends, sizeof a.ends);
-  a.dst = (const int *)(scratch + diag_bytes + pad_bytes);
-  a.sched = (const SchedWord *)(scratch + head_bytes);
+  const size_t word_bytes = ((size_t)L * Lc * sizeof(SchedWord) + 15) & ~(size_t)15;
+  unsigned char *d_words = scratch + diag_bytes + pad_bytes, *d_map = d_words + word_bytes;
+  a.dst = (const int *)d_map;
+  a.sched = (const SchedWord *)d_words;
   a.src = nullptr;  // only the global-memory A path reads it
   a.tol = tol; a.maxit = maxit; a.x0_given = 0; a.queue = nullptr;
   int wpb = 4;
@@ -2461,9 +2471,9 @@ camp_status camp_solve_noalloc(int n, int nnz, const int *row_ptr,
                            cudaMemcpyHostToDevice, st)) != cudaSuccess ||
       (e = cudaMemcpyAsync(scratch + diag_bytes, g_noalloc_padfrom, (size_t)Lc * sizeof(int),
                            cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(scratch + diag_bytes + pad_bytes, g_noalloc_dst,
-                           (size_t)nnz * sizeof(int), cudaMemcpyHostToDevice, st)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(scratch + head_bytes, g_noalloc_packed,
+      (e = cudaMemcpyAsync(d_map, g_noalloc_dst, (size_t)(dst_odd(nnz) + nnz) * sizeof(int),
+                           cudaMemcpyHostToDevice, st)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(d_words, g_noalloc_packed,
                            (size_t)L * Lc * sizeof(SchedWord), cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return cuda_fail(e, "staging into the static scratch");
   if ((e = launch_warp(E, a, wpb, grid, smem, st)) != cudaSuccess)

@@ -230,37 +230,38 @@ __device__ __forceinline__ void seg_spmv_gather(const SchedWord *__restrict__ sc
 }
 
 // Coalesced, vectorised read of one cell's A row (CSR order), handed to
-// put(slot, value) with the slot from the dst map.  The row is read in
+// put(place, value) with the place from the dst map.  The row is read in
 // 16-byte pairs from its first 16-byte boundary (lane sl reads pairs sl,
 // sl + Lc, ...); an entry before that boundary and an odd entry at the end
-// are read alone by lane 0.  The loads of kStagePairs pairs are issued before
-// any store, so a lane waits for memory once per batch rather than once per
-// entry.
+// are read alone by lane 0.  The map is kept twice, the copy at odd shifted by
+// one int, so that the pairs' places are 8-byte loads at either boundary.  The
+// loads of P pairs are issued before any store, so a lane waits for memory
+// once per batch rather than once per entry.
 constexpr int kStagePairs = 8;
-template <class Put>
+template <int P = kStagePairs, class Put>
 __device__ __forceinline__ void stage_scatter(const double *__restrict__ Ac,
                                               const int *__restrict__ dst, int nnz,
                                               int sl, int Lc, bool live, Put put) {
   const int h = (int)((reinterpret_cast<size_t>(Ac) >> 3) & 1);  // entries before the boundary
   const int np = (nnz - h) >> 1;                                  // whole pairs
   const double2 *A2 = reinterpret_cast<const double2 *>(Ac + h);
-  const int *d2 = dst + h;
-  for (int p0 = sl; p0 < np; p0 += kStagePairs * Lc) {
-    double2 v[kStagePairs];
-    int d[2 * kStagePairs];
+  const int2 *d2 = reinterpret_cast<const int2 *>(dst + (h ? dst_odd(nnz) + 1 : 0));
+  for (int p0 = sl; p0 < np; p0 += P * Lc) {
+    double2 v[P];
+    int2 d[P];
 #pragma unroll
-    for (int u = 0; u < kStagePairs; ++u) {
+    for (int u = 0; u < P; ++u) {
       const int p = p0 + u * Lc;
       const bool in = p < np;
-      d[2 * u] = in ? __ldg(d2 + 2 * p) : -1;
-      d[2 * u + 1] = in ? __ldg(d2 + 2 * p + 1) : -1;
+      d[u] = in ? __ldg(d2 + p) : make_int2(-1, -1);
       v[u] = (live && in) ? __ldg(A2 + p) : make_double2(0.0, 0.0);
     }
 #pragma unroll
-    for (int u = 0; u < kStagePairs; ++u) {
-      if (d[2 * u] >= 0) put(d[2 * u], v[u].x);
-      if (d[2 * u + 1] >= 0) put(d[2 * u + 1], v[u].y);
-    }
+    for (int u = 0; u < P; ++u)
+      if (d[u].x >= 0) {
+        put(d[u].x, v[u].x);
+        put(d[u].y, v[u].y);
+      }
   }
   if (sl == 0) {
     if (h) put(__ldg(dst), live ? __ldg(Ac) : 0.0);

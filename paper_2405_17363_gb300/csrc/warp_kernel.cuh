@@ -311,6 +311,13 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   st = -1;
   it = 0;
   resid = 0.0;
+  // the right-hand side's loads first: their latency runs beside the staging's
+  double r[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int i = sl + e * Lc;
+    r[e] = (live && i < n) ? (SRC == kSrcNewton ? nrh[i] : __ldg(a.b + (size_t)c * n + i)) : 0.0;
+  }
   // ---- stage the cell's matrix values in slot order (Sec. 3.1: one cell,
   // one team); the transposed view's permutation is folded into src
   if (SRC == kSrcAssembled || SRC == kSrcNewton) {
@@ -339,7 +346,7 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
   // r also holds s = r - alpha v between the half steps, and the true residual
   // at the end; what a segment that no longer iterates keeps in r, p and the
   // scalars is never read
-  double r[E], p[E];
+  double p[E];
   double bb;
   {
     double acc[1] = {0.0};
@@ -347,14 +354,12 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
     for (int e = 0; e < E; ++e) {
       const int i = sl + e * Lc;
       const bool v = live && i < n;
-      const double bi = v ? (SRC == kSrcNewton ? nrh[i] : __ldg(a.b + (size_t)c * n + i)) : 0.0;
       const double d = v ? (ASMEM ? Abase[__ldg(a.dslot + i)]
                                : __ldg(Ac + __ldg(a.dentry + i))) : 0.0;
       dvs[e] = v ? (!is_zero_bits(d) ? recip64(d) : 1.0) : 0.0;
       xv[e] = (v && a.x0_given) ? a.x[(size_t)c * n + i] : 0.0;
-      r[e] = bi;
       p[e] = 0.0;
-      acc[0] = fma(bi, bi, acc[0]);
+      acc[0] = fma(r[e], r[e], acc[0]);
     }
     bb = ssum1<LC>(acc[0], Lc);
   }

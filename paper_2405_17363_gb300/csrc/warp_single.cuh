@@ -75,6 +75,12 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
   double resid = 0.0;
   const bool live = has;
 
+  double r[E0], p[E0];  // r also holds s and the true residual, as in solve_group
+#pragma unroll
+  for (int j = 0; j < E0; ++j) {
+    const int i = row(j);
+    r[j] = live && j < EJ && i < n ? __ldg(a.b + (size_t)c * n + i) : 0.0;
+  }
   // ---- stage the cell's matrix values in split-slot order
   stage_scatter(Ac, a.dst2, nnz, lane, 32, live, [&](int t, double x) { Abase[t] = x; });
   zero_padding(Abase, a.pads2, a.npads2, a.L2, lane, 32);
@@ -85,7 +91,6 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
   }
   __syncwarp();
 
-  double r[E0], p[E0];  // r also holds s and the true residual, as in solve_group
   double bb;
   {
     double acc = 0.0;
@@ -93,11 +98,9 @@ __device__ __forceinline__ void solve_single(const WarpArgs &a, int pos, double 
     for (int j = 0; j < E0; ++j) {
       const int i = row(j);
       const bool ok = live && j < EJ && i < n;
-      const double bi = ok ? __ldg(a.b + (size_t)c * n + i) : 0.0;
       const double d = ok ? Abase[__ldg(a.dslot2 + i)] : 0.0;
       dvs[j] = ok ? (!is_zero_bits(d) ? recip64(d) : 1.0) : 0.0;
       xv[j] = (ok && a.x0_given) ? a.x[(size_t)c * n + i] : 0.0;
-      r[j] = bi;
       p[j] = 0.0;
       rhs[j] = 0.0;
     }
