@@ -643,8 +643,8 @@ __device__ __forceinline__ void plain_launch_body(const WarpArgs &a) {
         // a single-cell ticket: one cell on all 32 lanes (warp_single.cuh)
         const int ps = 2 * a.single_from + ((int)g - a.single_from);
         const bool one = a.ord_ws && lane == 0 && ps < a.cells;
-        if (one) wait_order_entry(a.order + ps, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
-        __syncwarp();
+        if (a.ord_ws)
+          wait_order_entries(a.order + ps, one, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
         solve_single<E>(a, ps, wbase);
         if (one) a.ord_out[ps] = 0;
         continue;
@@ -655,8 +655,8 @@ __device__ __forceinline__ void plain_launch_body(const WarpArgs &a) {
       // then clear them
       const int p = (int)g * k + lane;
       const bool mine = a.ord_ws && lane < k && p < a.cells;
-      if (mine) wait_order_entry(a.order + p, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
-      __syncwarp();
+      if (a.ord_ws)
+        wait_order_entries(a.order + p, mine, a.ord_ws + kOrdFlag, a.ord_err, a.ord_wait);
       solve_group<E, SRC, LC>(a, (int)g, wbase, sch_s);
       if (mine) a.ord_out[p] = 0;
     }
