@@ -30,7 +30,7 @@ __global__ void classify_kernel(const double *__restrict__ A, int cells, int n, 
     }
     worst = __reduce_max_sync(kFull, worst);
     if (lane == 0) {
-      const int k = difficulty_class(worst);
+      const int k = difficulty_class<kTopDeparture>(worst);
       cls[c] = (unsigned char)k;
       atomicAdd(counts + k, 1);
     }
@@ -82,7 +82,7 @@ __global__ void batch_classify_kernel(const BatchOrderArgs a) {
     }
     worst = __reduce_max_sync(kFull, worst);
     if (lane == 0) {
-      const int k = difficulty_class(worst);
+      const int k = difficulty_class<kTopDeparture>(worst);
       a.cls[i] = (unsigned char)k;
       atomicAdd(a.counts + m * 2 * kClasses + k, 1);
     }

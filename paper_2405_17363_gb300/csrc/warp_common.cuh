@@ -8,14 +8,20 @@ namespace camp {
 
 constexpr unsigned kFull = 0xffffffffu;
 
-// Difficulty class of a cell from the high word of its estimate
-// max_i |A_ii - 1| (a non-negative double, so its high words order as
-// integers): the half-octave index (exponent and first fraction bit),
-// largest first; estimates >= 12 share class 0, those below 2^-29 (and zero)
-// the last class.
+// Difficulty class of a cell from the high word of its estimate (a
+// non-negative double, so its high words order as integers): the half-octave
+// index (exponent and first fraction bit), largest first, 32 octaves down from
+// TOP.  max_i |A_ii - 1| takes TOP 2^19 (estimates from 3/2 2^19 share class 0,
+// those below 2^-12, which converge in an iteration or two, the last one): the
+// stiff cells of a long step have estimates of 10^2 to 10^5 and 15 to 300
+// iterations, and with 12 and above in one class they came in no order at all
+// (80 species x 4,000 such cells: 2,730 us; see below for the present figure).
+// |gamma| takes TOP 2^3.
+constexpr int kTopDeparture = 19, kTopGamma = 3;
+template <int TOP>
 __device__ __forceinline__ int difficulty_class(unsigned hi) {
   const int idx = (int)(hi >> 19);  // 2 * biased exponent + top fraction bit
-  const int top = ((1023 + 3) << 1) | 1;
+  const int top = ((1023 + TOP) << 1) | 1;
   const int c = top - idx;
   return c < 0 ? 0 : (c >= kOrdClasses ? kOrdClasses - 1 : c);
 }
@@ -690,7 +696,7 @@ __device__ __forceinline__ void order_prologue(const Args &a, int *sm) {
     __syncthreads();
     for (int i = threadIdx.x; i < pc; i += blockDim.x) {
       const unsigned long long kk = key[i];
-      const int k = difficulty_class((unsigned)(kk >> 32));
+      const int k = difficulty_class<BY_GAMMA ? kTopGamma : kTopDeparture>((unsigned)(kk >> 32));
       const int w = k | atomicAdd(hist + k, 1) << 6;
       if (a.ord_hits) atomicMax(bkey, kk);
       if (one_piece) key[i] = (unsigned)w;
