@@ -7,7 +7,7 @@
 // product must store and reset its running sum conditionally after every
 // multiply-add, and that select sits on the FP64 chain.  Here the rows are
 // packed again, into the same number of slots per lane, so that all lanes
-// end their rows in a few common slots (8 or 9 of 36 at 80 rows on 16 lanes):
+// end their rows in a few common slots (8 to 11 of 36 at 80 rows on 16 lanes):
 // the kernels run the others as bare multiply-adds.
 //
 // The common slots are found by a seeded random search over sets of m

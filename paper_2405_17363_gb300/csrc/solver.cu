@@ -806,8 +806,8 @@ camp_status ensure_order_capacity(camp_solver_t h, int cells, cudaStream_t st) {
 // Whether ordering the cells can shorten a launch: with at most one group per
 // SM sub-partition every group starts at once on an FP64 unit of its own, and
 // the launch ends with its hardest cell whatever the order, so the prologue
-// (and the cooperative launch) would only delay it (64 cells of 30 species: 36
-// us with it, 28 without; 600 cells of 80 species: 45 and 37).
+// (and the cooperative launch) would only delay it (64 cells of 30 species:
+// 35.6 us with it, 32.5 without; 600 cells of 80 species: 45.5 and 42.0).
 bool worth_ordering(camp_solver_t h, int ngroups) { return ngroups > 4 * h->sms; }
 
 // In-launch ordering of the fused-assembly and Newton launches (orderings 1
@@ -933,8 +933,8 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 // the last R pairs of the launch become 2R single-cell tickets.  Automatic R
 // (measured at 80 species on 152 SMs x 12 warps): every pair when the pairs
 // would keep at most three quarters of the resident warps busy (a lone warp's
-// latency decides such a launch: 49 against 62 us at 600 cells, 81 against 86
-// at 3,000, 108 against 91 at 4,000), a third when the launch shares the GPU
+// latency decides such a launch: 42 against 56 us at 600 cells, 77 against 83
+// at 3,000, but 103 against 87 at 4,000), a third when the launch shares the GPU
 // with others (`shared`: the chunks of the host-memory pipeline), else none
 // (at full load one cell per warp costs about 13 % more per cell).
 // camp_solver_set_single_tail overrides it.  Sets
@@ -1091,7 +1091,7 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
 extern "C" {
 
 const char *camp_last_error(void) { return g_err.c_str(); }
-const char *camp_version(void) { return "campsolve 0.17 (sm_103a)"; }
+const char *camp_version(void) { return "campsolve 0.18 (sm_103a)"; }
 
 camp_status camp_schedule_build(int n, int nnz, const int *row_ptr,
                                 const int *col_idx, int lanes_per_cell,

@@ -15,7 +15,8 @@ constexpr unsigned kFull = 0xffffffffu;
 // those below 2^-12, which converge in an iteration or two, the last one): the
 // stiff cells of a long step have estimates of 10^2 to 10^5 and 15 to 300
 // iterations, and with 12 and above in one class they came in no order at all
-// (80 species x 4,000 such cells: 2,730 us; see below for the present figure).
+// (80 species, pairs: 4,000 such cells 2,454 us, 2,235 in order; 6,000 cells
+// 3,549 and 3,012).
 // |gamma| takes TOP 2^3.
 constexpr int kTopDeparture = 19, kTopGamma = 3;
 template <int TOP>
@@ -124,11 +125,13 @@ __device__ __forceinline__ void slot_end(unsigned w, T &acc, unsigned os) {
 // which is also the sub-partition's issue interval) bounds both a lone warp
 // and a full SM, so everything else runs under it: the gathers and A values
 // of a half block are issued two multiply-adds ahead, the words a block
-// ahead, and only the slots of the end mask (8 or 9 of 36 at 80 rows on 16
+// ahead, and only the slots of the end mask (8 to 11 of 36 at 80 rows on 16
 // lanes) put a select on the chain.  Measured at 80 rows, 564 entries, 16
-// lanes: 76 cycles per slot for a lone warp against 100 with a conditional
-// store and select in every slot, 65 per slot and warp with four warps per
-// sub-partition either way.
+// lanes, in isolation: 95 cycles per slot for a lone warp against 100 with a
+// conditional store and select in every slot, in 520 instructions against 915;
+// 65 per slot and warp with three or four warps per sub-partition either way.
+// (Two word sets and an unrolled pair of blocks: 81 alone, but the kernels
+// around it spilled: 183 us against 180 at 80 species x 10,000 cells.)
 template <class T, class Lo, class Hi, class Last>
 __device__ __forceinline__ void spmv_slots(const SchedWord *__restrict__ sch,
                                            const unsigned *__restrict__ ends, int L, int Lc, int sl,

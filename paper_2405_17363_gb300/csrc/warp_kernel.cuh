@@ -91,9 +91,11 @@ __device__ __forceinline__ void table_constants(const WarpArgs &a, double *Abase
 
 // A = I - gamma J(conc), every entry by the chain of multiply-adds of its
 // terms and one for the identity part (ab: shared address of the matrix
-// block).  FP64-bound: 42 + 36 multiply-adds per lane at 80 species, 200
-// reactions, 16 lanes, against 65 + 36 with every lane summing the terms of its
-// own slots in shared memory.
+// block).  FP64-bound: 41 + 36 multiply-adds per lane at 80 species, 200
+// reactions, 16 lanes.  With every lane summing the terms of its own slots in
+// shared memory the fullest lane set the pace: assembly + solve of 10,000 cells
+// took 206 us against 204, the Newton corrector 603 against 559 (with the rates
+// below).
 __device__ __forceinline__ void assemble_matrix(const MechTables &m, unsigned ab, double gam,
                                                 int sl, int Lc) {
   const int4 *head = m.jhead + sl, *step = m.jstep + sl;
