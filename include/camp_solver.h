@@ -287,8 +287,9 @@ camp_status camp_batch_set_config(camp_batch_t b, int rows_per_lane,
  * 1 (default) hands each mechanism's cells to warps hardest first, by the
  * same difficulty estimate and classes as camp_solver_set_ordering (a
  * classify and a scatter launch over all mechanisms, part of the batch's
- * graph; device scratch of 5 bytes per cell plus 512 bytes per mechanism);
- * 0 keeps index order.  Results are bitwise the same either way.
+ * graph; device scratch of 9 bytes per cell plus 256 bytes per mechanism);
+ * 0 keeps index order, as does a batch with at most one work item per SM
+ * sub-partition.  Results are bitwise the same either way.
  * CAMP_EINVAL for other values.
  */
 camp_status camp_batch_set_ordering(camp_batch_t b, int ordering);

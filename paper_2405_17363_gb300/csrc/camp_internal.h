@@ -240,7 +240,8 @@ cudaError_t launch_difficulty_order(const double *A, int cells, int n, int nnz,
 // Difficulty ordering of a persistent multi-mechanism batch (order.cu): one
 // classify and one scatter launch over the concatenated cells of all
 // mechanisms (cell_begin: offsets, cell_begin[nmech] = total); counts holds
-// per mechanism kOrdClasses totals then kOrdClasses cursors (zero on entry);
+// per mechanism kOrdClasses totals (zero on entry), cls and pos a cell's class
+// and its place in it;
 // order + cell_begin[m] receives mechanism m's cells, hardest class first.
 struct BatchOrderArgs {
   int nmech;
@@ -250,8 +251,9 @@ struct BatchOrderArgs {
   int cell_begin[kMaxMech + 1];
   unsigned char *cls;
   int *counts;
-  int *order;
+  int *order, *pos;
 };
+constexpr int kBatchOrderPiece = 64;  // cells a block of the classify launch takes
 const void *batch_classify_kernel_fn();  // __global__ (const BatchOrderArgs)
 const void *batch_scatter_kernel_fn();   // __global__ (const BatchOrderArgs), 1 thread per cell
 

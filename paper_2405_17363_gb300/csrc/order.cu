@@ -65,13 +65,24 @@ __global__ void scatter_kernel(const unsigned char *__restrict__ cls, int cells,
 // The same two steps for the persistent multi-mechanism batch, all
 // mechanisms in one launch each: cell i of the concatenated cell space
 // belongs to mechanism m with cell_begin[m] <= i < cell_begin[m + 1]; every
-// mechanism has its own class totals and cursors (counts + m * 2 kClasses)
-// and its own order (order + cell_begin[m], cell indices within m).
+// mechanism has its own class totals (counts + m kClasses) and its own order
+// (order + cell_begin[m], cell indices within m).  A block classifies
+// kBatchOrderPiece consecutive cells, counts them in shared memory and reserves
+// its range of every class with one atomic, so the scatter needs none; with a
+// global atomic per cell in either launch the batch of 25,500 cells took 317 us
+// instead of 314.
 __global__ void batch_classify_kernel(const BatchOrderArgs a) {
-  const int lane = threadIdx.x & 31;
-  const int warps = (gridDim.x * blockDim.x) >> 5;
+  __shared__ int hist[kMaxMech * kClasses], base[kMaxMech * kClasses];
+  __shared__ int slot[kBatchOrderPiece], rank[kBatchOrderPiece];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
   const int total = a.cell_begin[a.nmech];
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < total; i += warps) {
+  const int i0 = blockIdx.x * kBatchOrderPiece;
+  for (int q = threadIdx.x; q < kMaxMech * kClasses; q += blockDim.x) hist[q] = 0;
+  __syncthreads();
+#pragma unroll 2
+  for (int j = warp; j < kBatchOrderPiece; j += warps) {
+    const int i = i0 + j;
+    if (i >= total) break;
     int m = 0;
     while (m + 1 < a.nmech && i >= a.cell_begin[m + 1]) ++m;
     const double *Ac = a.A[m] + (size_t)(i - a.cell_begin[m]) * a.nnz[m];
@@ -82,18 +93,26 @@ __global__ void batch_classify_kernel(const BatchOrderArgs a) {
     }
     worst = __reduce_max_sync(kFull, worst);
     if (lane == 0) {
-      const int k = difficulty_class<kTopDeparture>(worst);
-      a.cls[i] = (unsigned char)k;
-      atomicAdd(a.counts + m * 2 * kClasses + k, 1);
+      slot[j] = m * kClasses + difficulty_class<kTopDeparture>(worst);
+      rank[j] = atomicAdd(hist + slot[j], 1);
     }
   }
+  __syncthreads();
+  for (int q = threadIdx.x; q < a.nmech * kClasses; q += blockDim.x)
+    if (hist[q]) base[q] = atomicAdd(a.counts + q, hist[q]);
+  __syncthreads();
+  for (int j = threadIdx.x; j < kBatchOrderPiece; j += blockDim.x)
+    if (i0 + j < total) {
+      a.cls[i0 + j] = (unsigned char)(slot[j] % kClasses);
+      a.pos[i0 + j] = base[slot[j]] + rank[j];
+    }
 }
 
 __global__ void batch_scatter_kernel(const BatchOrderArgs a) {
   __shared__ int start[kMaxMech][kClasses];
   for (int m = threadIdx.x >> 5; m < a.nmech; m += blockDim.x >> 5) {
     const int l = threadIdx.x & 31;
-    const int *cnt = a.counts + m * 2 * kClasses;
+    const int *cnt = a.counts + m * kClasses;
     const int x = cnt[2 * l], y = cnt[2 * l + 1];
     int s = x + y;
 #pragma unroll
@@ -109,9 +128,7 @@ __global__ void batch_scatter_kernel(const BatchOrderArgs a) {
   if (i < a.cell_begin[a.nmech]) {
     int m = 0;
     while (m + 1 < a.nmech && i >= a.cell_begin[m + 1]) ++m;
-    const int k = a.cls[i];
-    const int pos = start[m][k] + atomicAdd(a.counts + m * 2 * kClasses + kClasses + k, 1);
-    a.order[a.cell_begin[m] + pos] = i - a.cell_begin[m];
+    a.order[a.cell_begin[m] + start[m][a.cls[i]] + a.pos[i]] = i - a.cell_begin[m];
   }
 }
 

@@ -2174,25 +2174,28 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
     oa.cell_begin[q + 1] = oa.cell_begin[q] + cells[m];
   }
   const int total_cells = oa.cell_begin[b->nmech];
-  const bool ordered = b->ordering && total_cells > 1;
-  const size_t cnt_bytes = (size_t)b->nmech * 2 * kOrdClasses * sizeof(int);
+  // (see worth_ordering: with every item running at once the order is no use,
+  // and its three nodes come before the solve)
+  const bool ordered = b->ordering && items > 4 * b->sms;
+  const size_t cnt_bytes = (size_t)b->nmech * kOrdClasses * sizeof(int);
   if (ordered) {
     if ((size_t)total_cells > b->ord_cap) {
       cudaFree(b->d_ord);
       b->d_ord = nullptr;
       b->ord_cap = 0;
-      // counters, the order (4 bytes per cell), then the classes (1 byte per cell)
-      if ((e = cudaMalloc(&b->d_ord, cnt_bytes + (size_t)total_cells * 5)) != cudaSuccess)
+      // counters, the order and the places (4 bytes per cell each), then the
+      // classes (1 byte per cell)
+      if ((e = cudaMalloc(&b->d_ord, cnt_bytes + (size_t)total_cells * 9)) != cudaSuccess)
         return fail(CAMP_ENOMEM, "batch ordering scratch: %s", cudaGetErrorString(e));
       b->ord_cap = (size_t)total_cells;
     }
     oa.counts = (int *)b->d_ord;
     oa.order = (int *)(b->d_ord + cnt_bytes);
-    oa.cls = b->d_ord + cnt_bytes + b->ord_cap * 4;
+    oa.pos = oa.order + b->ord_cap;
+    oa.cls = b->d_ord + cnt_bytes + b->ord_cap * 8;
     for (int q = 0; q < b->nmech; ++q) args.m[q].order = oa.order + oa.cell_begin[q];
   }
-  const int ogrid = (int)std::max(1L, std::min(((long)total_cells * 32 + 255) / 256,
-                                                (long)b->sms * 8));
+  const int ogrid = std::max(1, (total_cells + kBatchOrderPiece - 1) / kBatchOrderPiece);
   const int sgrid = (total_cells + 255) / 256;
   void *oparams[] = {&oa};
   int wpb = b->wpb > 0 ? b->wpb : 4;
