@@ -346,7 +346,8 @@ struct MixedArgs {
 // inner iteration share; rounded to 16 and, with several cells per warp, to Lc
 // four-byte banks modulo the 32 (at least 16 bytes), so that the warp's cells
 // gather from different banks (24 species, 8 lanes: a multiple of 128 bytes
-// put all four cells of a warp on the same ones).
+// put all four cells of a warp on the same ones, 254 us against 211 for 88,758
+// cells).
 __host__ __device__ inline size_t mixed_cell_bytes(int segA, int segV, bool a64_smem, int Lc) {
   const size_t need = ((size_t)(a64_smem ? 12 : 4) * segA + (size_t)16 * segV + 15) & ~(size_t)15;
   if (Lc >= 32) return need;

@@ -525,8 +525,13 @@ sched::RowChains row_chains(const Schedule &S, const std::vector<int> &rp) {
 }
 
 // A layout of the view's rows at Lc lanes per cell.  Every row keeps the
-// entry order of its Lc-lane schedule in each, so its sum keeps its bits.
-cudaError_t view_schedule(View &v, int Lc, Kind kind, Layout **out, const Slots **slots) {
+// entry order of its Lc-lane schedule in each, so its sum keeps its bits.  A
+// layout cannot be built while st captures a graph (it allocates): the plain and
+// the aligned layout then stand in for each other, and a missing kOne is
+// returned empty (L 0), so a call whose lane count has been used before still
+// captures.
+cudaError_t view_schedule(View &v, int Lc, Kind kind, cudaStream_t st, Layout **out,
+                          const Slots **slots) {
   auto it = v.sched.find(Lc);
   if (it == v.sched.end()) {
     it = v.sched.emplace(Lc, Layout()).first;
@@ -537,6 +542,14 @@ cudaError_t view_schedule(View &v, int Lc, Kind kind, Layout **out, const Slots 
   if (out) *out = &Y;
   *slots = &to;
   if (to.L) return cudaSuccess;
+  const Slots &other = Y.slots[kind == kPlain ? kAligned : kPlain];
+  if (kind == kOne || other.L) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) {
+      if (kind != kOne) *slots = &other;
+      return cudaSuccess;
+    }
+  }
   Schedule &S = Y.base;
   std::vector<int> dentry(v.n);
   for (int i = 0; i < v.n; ++i) dentry[i] = S.src[S.dslot[i]];
@@ -942,7 +955,7 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 // the launch without single tickets when the split schedule does not fit
 // the warp's region.
 cudaError_t set_single_tickets(camp_solver_t h, View &v, WarpArgs &a, int wpb, int occ,
-                               bool shared) {
+                               bool shared, cudaStream_t st) {
   const int pairs = a.ngroups;
   a.single_from = pairs;
   a.sched2 = nullptr;
@@ -957,11 +970,11 @@ cudaError_t set_single_tickets(camp_solver_t h, View &v, WarpArgs &a, int wpb, i
   }
   if (R == 0) return cudaSuccess;
   const Slots *S = nullptr;
-  const cudaError_t e = view_schedule(v, 16, kOne, nullptr, &S);
+  const cudaError_t e = view_schedule(v, 16, kOne, st, nullptr, &S);
   if (e != cudaSuccess) return e;
   const size_t need =
       ((size_t)(S->L * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
-  if (need > 2 * (size_t)a.segStride) return cudaSuccess;
+  if (S->L == 0 || need > 2 * (size_t)a.segStride) return cudaSuccess;
   const int P = pairs - R;
   a.single_from = P;
   a.ngroups = P + std::max(0, a.cells - 2 * P);
@@ -1006,7 +1019,7 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
                   v.n, E, Lc, kMaxE);
     Layout *Y = nullptr;
     const Slots *S = nullptr;
-    e = view_schedule(v, Lc, kAligned, &Y, &S);
+    e = view_schedule(v, Lc, kAligned, st, &Y, &S);
     if (e != cudaSuccess) return cuda_fail(e, "schedule upload");
     int wpb = h->wpb > 0 ? h->wpb : 4;
     int segA = 0, segV = 0, segStride = 0;
@@ -1039,7 +1052,7 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
     e = warp_occupancy(E, Lc, kTicketsPack, wpb, smem, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy");
     if (occ < 1) occ = 1;
-    if ((e = set_single_tickets(h, v, a, wpb, occ, queue_slot != 0)) != cudaSuccess)
+    if ((e = set_single_tickets(h, v, a, wpb, occ, queue_slot != 0, st)) != cudaSuccess)
       return cuda_fail(e, "schedule upload");
     if (tickets_of(a) != kTicketsPack) {
       e = warp_occupancy(E, Lc, tickets_of(a), wpb, smem, &occ);
@@ -1786,7 +1799,7 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
     return fail(CAMP_EUNSUPPORTED, "fused assembly supports at most 8 rows per lane (n=%d)", v.n);
   Layout *Y = nullptr;
   const Slots *S = nullptr;
-  if ((e = view_schedule(v, Lc, kAligned, &Y, &S)) != cudaSuccess)
+  if ((e = view_schedule(v, Lc, kAligned, h->stream, &Y, &S)) != cudaSuccess)
     return cuda_fail(e, "schedule upload");
   if (S->L > 2047) return fail(CAMP_EUNSUPPORTED, "more than 2047 slots per lane");
   MechTerms *T = nullptr;
@@ -1927,7 +1940,7 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
   const int E = (v.n + Lc - 1) / Lc;
   if (E > kMaxE) return fail(CAMP_EUNSUPPORTED, "n=%d too large for %d lanes per cell", v.n, Lc);
   const Slots *S = nullptr;
-  if ((e = view_schedule(v, Lc, kPlain, nullptr, &S)) != cudaSuccess)
+  if ((e = view_schedule(v, Lc, kPlain, h->stream, nullptr, &S)) != cudaSuccess)
     return cuda_fail(e, "schedule upload");
   // FP64 A in shared memory unless that costs resident warps (then the
   // outer residual product reads it through L1)
@@ -2139,7 +2152,7 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
     int Lc = 1;
     while ((v.n + Lc - 1) / Lc > E) Lc *= 2;
     const Slots *S = nullptr;
-    if ((e = view_schedule(v, Lc, kAligned, nullptr, &S)) != cudaSuccess)
+    if ((e = view_schedule(v, Lc, kAligned, b->stream, nullptr, &S)) != cudaSuccess)
       return cuda_fail(e, "schedule upload");
     WarpArgs &a = args.m[q];
     a.cells = cells[m]; a.n = v.n; a.nnz = v.nnz;

@@ -337,3 +337,36 @@ def test_large_batch_all_cells(camp, cuda):
     assert np.all(gpu["status"] == 0) and np.all(gpu["resid"] <= tol)
     orc = oracle.solve(m.row_ptr, m.col_idx, cb.A_vals, cb.b, tol, maxit, threads=THREADS)
     parity.compare(m, cb.A_vals, cb.b, tol, gpu, orc, "480k")
+
+
+@pytest.mark.parametrize("n,R", [(80, 200), (90, 210)])
+def test_capture_of_another_route_after_one_solve(camp, cuda, n, R):
+    """One large solve prepares the handle; a small batch (single cells on a warp
+    at 80 species) and the refinement (the same lane count at 90 species) can then
+    be captured, though their layouts were never needed: replays give bitwise the
+    eager results."""
+    import torch
+    m = synth.make_mechanism(n, R, 77)
+    cb = synth.make_cells(m, 5000, 78, gamma=(1e-4, 1e-1))
+    A, b = to_dev(cb.A_vals, cuda), to_dev(cb.b, cuda)
+    ref = camp.Solver(m.row_ptr, m.col_idx)
+    want = [t.clone() for t in ref.solve(A[:64], b[:64])]
+    wmix = [t.clone() for t in ref.solve_mixed(A[:64], b[:64])]
+    s = camp.Solver(m.row_ptr, m.col_idx)
+    s.solve(A, b)
+    mixed = n > 80   # the refinement takes 32 lanes, as the solve does above 80 species
+    out = [torch.empty_like(t) for t in want]
+    omix = [torch.empty_like(t) for t in wmix]
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        s.solve(A[:64], b[:64], out=out)
+        if mixed:
+            s.solve_mixed(A[:64], b[:64], out=omix)
+    g.replay()
+    torch.cuda.synchronize()
+    for x, y in zip(want + (wmix if mixed else []), out + (omix if mixed else [])):
+        assert torch.equal(x, y)
+    del g
+    s.close()
+    ref.close()
