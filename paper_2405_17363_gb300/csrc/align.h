@@ -106,11 +106,12 @@ inline int align(int n, const RowChains &ch, int Lc, int max_slots, std::vector<
   unsigned seed = 12345u;
   std::vector<int> found;
   const int m0 = (n + Lc - 1) / Lc;  // rows of a lane
+  int tries = 480;  // bounds the search for patterns that have no such layout
   for (int L = fewest; L <= max_slots && found.empty(); ++L)
     for (int m = std::min(L, m0 + 3); m <= std::min(L, m0 + 9) && found.empty(); m += 2) {
       std::vector<int> base, pos;
       int best = n + 1;
-      for (int t = 0; t < 40 && found.empty(); ++t) {
+      for (int t = 0; t < 40 && found.empty() && tries > 0; ++t, --tries) {
         std::vector<char> is(L + 1, 0);
         if (base.empty() || next_random(seed) % 10 == 0) {
           for (int c = 0; c < m - 1;) {
