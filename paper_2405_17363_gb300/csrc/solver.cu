@@ -10,6 +10,8 @@
 #include <mutex>
 #include <numeric>
 #include <string>
+#include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "camp_internal.h"
@@ -334,12 +336,8 @@ struct Slots {
   int *d_dst = nullptr, *d_dslot = nullptr, *d_pads = nullptr;        // pair_pos places
   int *d_dst32 = nullptr, *d_dslot32 = nullptr, *d_pads32 = nullptr;  // word_pos places
   int *d_dentry = nullptr;   // [n] A entry of each row's diagonal
-  void release() {
-    for (void *p : {(void *)d_words, (void *)d_src, (void *)d_dst, (void *)d_dslot,
-                    (void *)d_pads, (void *)d_dst32, (void *)d_dslot32, (void *)d_pads32,
-                    (void *)d_dentry})
-      cudaFree(p);
-  }
+  void *block = nullptr;     // holds them all
+  void release() { cudaFree(block); }
 };
 
 // The layouts of one lane count, each built when first used (L 0: not yet).
@@ -364,15 +362,39 @@ struct View {
   std::map<int, Layout> sched;  // by lanes per cell
 };
 
-template <class T>
-cudaError_t upload(T **dst, const std::vector<T> &src) {
-  *dst = nullptr;
-  if (src.empty()) return cudaSuccess;
-  cudaError_t e = cudaMalloc((void **)dst, src.size() * sizeof(T));
-  if (e != cudaSuccess) return e;
-  return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T),
-                    cudaMemcpyHostToDevice);
-}
+// Host tables on their way to the device: one block, one copy, on the device
+// when commit returns.  cudaMemcpy from pageable memory may return before its
+// data is there, and only streams ordered behind the legacy stream wait for it;
+// the kernels that read the tables run on any stream (solve_host's own and
+// PyTorch's side streams are not), so commit waits for the copy itself.
+class Upload {
+  std::vector<unsigned char> bytes;
+  std::vector<std::pair<void **, size_t>> at;
+
+ public:
+  template <class P, class T>
+  void add(P **dst, const std::vector<T> &src) {
+    static_assert(std::is_same_v<std::remove_const_t<P>, T>);
+    const size_t off = (bytes.size() + 255) & ~(size_t)255;  // as cudaMalloc aligns
+    bytes.resize(off + src.size() * sizeof(T));
+    if (!src.empty()) memcpy(bytes.data() + off, src.data(), src.size() * sizeof(T));
+    at.emplace_back((void **)dst, off);
+  }
+  cudaError_t commit(void **block) {
+    *block = nullptr;
+    cudaError_t e = cudaMalloc(block, std::max<size_t>(bytes.size(), 1));
+    if (e == cudaSuccess && !bytes.empty())
+      e = cudaMemcpy(*block, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+      cudaFree(*block);
+      *block = nullptr;
+      return e;
+    }
+    for (auto &a : at) *a.first = (unsigned char *)*block + a.second;
+    return e;
+  }
+};
 
 // Mass-action mechanism attached to a handle for the fused assembly: its
 // Jacobian terms in reaction order (pattern entry, concentration factor,
@@ -380,12 +402,8 @@ cudaError_t upload(T **dst, const std::vector<T> &src) {
 // per lanes-per-cell choice, their tables on the device.
 struct MechTerms {
   MechTables t = {};
-  void release() {
-    for (const void *p : {(const void *)t.jrun, (const void *)t.jhead, (const void *)t.jstep,
-                          (const void *)t.rchunk, (const void *)t.rate, (const void *)t.rrun,
-                          (const void *)t.rhead, (const void *)t.rstep})
-      cudaFree(const_cast<void *>(p));
-  }
+  void *block = nullptr;  // holds the tables
+  void release() { cudaFree(block); }
 };
 struct Mechanism {
   int R = 0;
@@ -410,6 +428,7 @@ struct camp_solver {
   cudaStream_t stream = nullptr;
   View fwd, tr;
   int *d_row_of = nullptr;  // forward view: row of entry k
+  void *d_block = nullptr;  // holds the views' arrays, d_row_of and d_queue
   // dynamic group queues of the warp kernel, one pair per stream the handle
   // uses: pair 0 its own stream, pairs 1.. the solve streams of solve_host
   unsigned int *d_queue = nullptr;
@@ -488,21 +507,22 @@ cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<uns
     dslot[i] = dst[dentry[i]];
     dslot32[i] = dst32[dentry[i]];
   }
-  cudaError_t e = upload(&S.d_words, words);
-  if (e == cudaSuccess) e = upload(&S.d_src, psrc);
   auto twice = [nnz](std::vector<int> v) {
     v.resize((size_t)dst_odd(nnz) + nnz);
     std::copy(v.begin(), v.begin() + nnz, v.begin() + dst_odd(nnz));
     return v;
   };
-  if (e == cudaSuccess) e = upload(&S.d_dst, twice(dst));
-  if (e == cudaSuccess) e = upload(&S.d_dslot, dslot);
-  if (e == cudaSuccess) e = upload(&S.d_pads, pads);
-  if (e == cudaSuccess) e = upload(&S.d_dst32, twice(dst32));
-  if (e == cudaSuccess) e = upload(&S.d_dslot32, dslot32);
-  if (e == cudaSuccess) e = upload(&S.d_pads32, pads32);
-  if (e == cudaSuccess) e = upload(&S.d_dentry, dentry);
-  return e;
+  Upload up;
+  up.add(&S.d_words, words);
+  up.add(&S.d_src, psrc);
+  up.add(&S.d_dst, twice(dst));
+  up.add(&S.d_dslot, dslot);
+  up.add(&S.d_pads, pads);
+  up.add(&S.d_dst32, twice(dst32));
+  up.add(&S.d_dslot32, dslot32);
+  up.add(&S.d_pads32, pads32);
+  up.add(&S.d_dentry, dentry);
+  return up.commit(&S.block);
 }
 
 // Every row's entries in the order of the schedule S.
@@ -572,18 +592,11 @@ cudaError_t view_schedule(View &v, int Lc, Kind kind, cudaStream_t st, Layout **
     src = S.src;
   }
   const cudaError_t e = upload_slots(to, lanes, L, v.nnz, word, src, dentry);
-  if (e != cudaSuccess) {
-    to.release();
-    to = Slots();
-  }
+  if (e != cudaSuccess) to = Slots();
   return e;
 }
 
 void free_view(View &v) {
-  cudaFree(v.d_rp);
-  cudaFree(v.d_ci);
-  cudaFree(v.d_diag);
-  cudaFree(v.d_perm);
   for (auto &kv : v.sched)
     for (Slots &S : kv.second.slots) S.release();
   v.sched.clear();
@@ -1271,20 +1284,17 @@ camp_status camp_solver_create(camp_solver_t *out, int n, int nnz,
   std::vector<int> row_of(nnz);
   for (int i = 0; i < n; ++i)
     for (int k = row_ptr[i]; k < row_ptr[i + 1]; ++k) row_of[k] = i;
-  if ((e = upload(&f.d_rp, f.rp)) != cudaSuccess ||
-      (e = upload(&f.d_ci, f.ci)) != cudaSuccess ||
-      (e = upload(&f.d_diag, f.diag)) != cudaSuccess ||
-      (e = upload(&t.d_rp, t.rp)) != cudaSuccess ||
-      (e = upload(&t.d_ci, t.ci)) != cudaSuccess ||
-      (e = upload(&t.d_diag, t.diag)) != cudaSuccess ||
-      (e = upload(&t.d_perm, t.perm)) != cudaSuccess ||
-      (e = upload(&h->d_row_of, row_of)) != cudaSuccess ||
-      (e = upload(&h->d_queue, std::vector<unsigned int>(2 * (1 + kHostSolveStreams) + kOrdWords,
-                                                          0u))) != cudaSuccess) {
-    free_view(h->fwd);
-    free_view(h->tr);
-    cudaFree(h->d_row_of);
-    cudaFree(h->d_queue);
+  Upload up;
+  up.add(&f.d_rp, f.rp);
+  up.add(&f.d_ci, f.ci);
+  up.add(&f.d_diag, f.diag);
+  up.add(&t.d_rp, t.rp);
+  up.add(&t.d_ci, t.ci);
+  up.add(&t.d_diag, t.diag);
+  up.add(&t.d_perm, t.perm);
+  up.add(&h->d_row_of, row_of);
+  up.add(&h->d_queue, std::vector<unsigned int>(2 * (1 + kHostSolveStreams) + kOrdWords, 0u));
+  if ((e = up.commit(&h->d_block)) != cudaSuccess) {
     delete h;
     return cuda_fail(e, "pattern upload");
   }
@@ -1299,8 +1309,7 @@ camp_status camp_solver_destroy(camp_solver_t h) {
   free_view(h->fwd);
   free_view(h->tr);
   for (auto &kv : h->mech.by_lanes) kv.second.release();
-  cudaFree(h->d_row_of);
-  cudaFree(h->d_queue);
+  cudaFree(h->d_block);
   cudaFree(h->d_order_scratch);
   if (h->h_ord_err) cudaFreeHost(h->h_ord_err);
   if (h->h_hits) cudaFreeHost(h->h_hits);
@@ -1765,20 +1774,17 @@ cudaError_t mech_terms(Mechanism &mech, int n, int Lc, const Slots &S, MechTerms
   MechTerms T;
   T.t.jruns = (int)J.runs.size();
   T.t.rchunks = (int)rchunk.size();
-  auto put = [](auto &dst, const auto &src) {
-    auto *p = const_cast<std::remove_const_t<std::remove_pointer_t<std::decay_t<decltype(dst)>>> *>(dst);
-    const cudaError_t e = upload(&p, src);
-    dst = p;
-    return e;
-  };
-  cudaError_t e;
-  if ((e = put(T.t.jrun, J.runs)) != cudaSuccess || (e = put(T.t.jhead, jhead)) != cudaSuccess ||
-      (e = put(T.t.jstep, jstep)) != cudaSuccess || (e = put(T.t.rchunk, rchunk)) != cudaSuccess ||
-      (e = put(T.t.rate, rate)) != cudaSuccess || (e = put(T.t.rrun, rrun)) != cudaSuccess ||
-      (e = put(T.t.rhead, rhead)) != cudaSuccess || (e = put(T.t.rstep, rstep)) != cudaSuccess) {
-    T.release();
-    return e;
-  }
+  Upload up;
+  up.add(&T.t.jrun, J.runs);
+  up.add(&T.t.jhead, jhead);
+  up.add(&T.t.jstep, jstep);
+  up.add(&T.t.rchunk, rchunk);
+  up.add(&T.t.rate, rate);
+  up.add(&T.t.rrun, rrun);
+  up.add(&T.t.rhead, rhead);
+  up.add(&T.t.rstep, rstep);
+  const cudaError_t e = up.commit(&T.block);
+  if (e != cudaSuccess) return e;
   *out = &mech.by_lanes.emplace(Lc, T).first->second;
   return cudaSuccess;
 }
