@@ -336,11 +336,13 @@ struct Slots {
   int *d_dst = nullptr, *d_dslot = nullptr, *d_pads = nullptr;        // pair_pos places
   int *d_dst32 = nullptr, *d_dslot32 = nullptr, *d_pads32 = nullptr;  // word_pos places
   int *d_dentry = nullptr;   // [n] A entry of each row's diagonal
-  void *block = nullptr;     // holds them all
-  void release() { cudaFree(block); }
 };
 
-// The layouts of one lane count, each built when first used (L 0: not yet).
+// The layouts of one lane count.  The plain and the aligned one are built
+// together when the lane count is first used, so which of them a call runs
+// never depends on the calls before it, or on whether its stream captures a
+// graph (where nothing can be allocated); kOne when a small batch first needs
+// it (L 0: not yet).
 enum Kind {
   kPlain = 0,    // the schedule as built (the refinement kernel)
   kAligned = 1,  // its rows aligned (align.h), where that takes no more slots
@@ -349,6 +351,7 @@ enum Kind {
 struct Layout {
   Schedule base;
   Slots slots[3];
+  void *block = nullptr, *block_one = nullptr;  // the slots' device arrays
   // automatic warps per block, found once per kernel kind (0: not yet):
   // plain solve, fused assembly, Newton corrector
   int auto_wpb[3] = {0, 0, 0};
@@ -475,10 +478,10 @@ struct camp_solver {
 
 namespace {
 
-// The device form of the slots word/src [L][Lc] (host words, A entry or -1);
-// dentry: the A entry of every row's diagonal.
-cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<unsigned> &word,
-                         const std::vector<int> &src, const std::vector<int> &dentry) {
+// The device form of the slots word/src [L][Lc] (host words, A entry or -1),
+// added to the upload; dentry: the A entry of every row's diagonal.
+void add_slots(Slots &S, Upload &up, int Lc, int L, int nnz, const std::vector<unsigned> &word,
+               const std::vector<int> &src, const std::vector<int> &dentry) {
   S.Lc = Lc;
   S.L = L;
   S.dentry = dentry;
@@ -512,7 +515,6 @@ cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<uns
     std::copy(v.begin(), v.begin() + nnz, v.begin() + dst_odd(nnz));
     return v;
   };
-  Upload up;
   up.add(&S.d_words, words);
   up.add(&S.d_src, psrc);
   up.add(&S.d_dst, twice(dst));
@@ -522,7 +524,6 @@ cudaError_t upload_slots(Slots &S, int Lc, int L, int nnz, const std::vector<uns
   up.add(&S.d_dslot32, dslot32);
   up.add(&S.d_pads32, pads32);
   up.add(&S.d_dentry, dentry);
-  return up.commit(&S.block);
 }
 
 // Every row's entries in the order of the schedule S.
@@ -544,61 +545,64 @@ sched::RowChains row_chains(const Schedule &S, const std::vector<int> &rp) {
   return ch;
 }
 
-// A layout of the view's rows at Lc lanes per cell.  Every row keeps the
-// entry order of its Lc-lane schedule in each, so its sum keeps its bits.  A
-// layout cannot be built while st captures a graph (it allocates): the plain and
-// the aligned layout then stand in for each other, and a missing kOne is
-// returned empty (L 0), so a call whose lane count has been used before still
-// captures.
-cudaError_t view_schedule(View &v, int Lc, Kind kind, cudaStream_t st, Layout **out,
-                          const Slots **slots) {
+// The layouts of the view's rows at Lc lanes per cell.  Every row keeps the
+// entry order of its Lc-lane schedule in each, so its sum keeps its bits.
+cudaError_t view_schedule(View &v, int Lc, Layout **out) {
   auto it = v.sched.find(Lc);
   if (it == v.sched.end()) {
-    it = v.sched.emplace(Lc, Layout()).first;
-    it->second.base = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
+    Layout Y;
+    Y.base = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
+    const Schedule &S = Y.base;
+    std::vector<int> dentry(v.n);
+    for (int i = 0; i < v.n; ++i) dentry[i] = S.src[S.dslot[i]];
+    std::vector<unsigned> word;
+    std::vector<int> src;
+    const int L = sched::align(v.n, row_chains(S, v.rp), Lc, S.L, word, src);
+    Upload up;
+    add_slots(Y.slots[kPlain], up, Lc, S.L, v.nnz, S.words, S.src, dentry);
+    if (L) add_slots(Y.slots[kAligned], up, Lc, L, v.nnz, word, src, dentry);
+    const cudaError_t e = up.commit(&Y.block);
+    if (e != cudaSuccess) return e;
+    if (!L) Y.slots[kAligned] = Y.slots[kPlain];
+    it = v.sched.emplace(Lc, std::move(Y)).first;
   }
-  Layout &Y = it->second;
-  Slots &to = Y.slots[kind];
-  if (out) *out = &Y;
+  *out = &it->second;
+  return cudaSuccess;
+}
+
+// The layout of a cell alone on 32 lanes; left empty (L 0) while st captures
+// a graph.
+cudaError_t one_slots(const View &v, Layout &Y, cudaStream_t st, const Slots **slots) {
+  Slots &to = Y.slots[kOne];
   *slots = &to;
   if (to.L) return cudaSuccess;
-  const Slots &other = Y.slots[kind == kPlain ? kAligned : kPlain];
-  if (kind == kOne || other.L) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone) {
-      if (kind != kOne) *slots = &other;
-      return cudaSuccess;
-    }
-  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
+    return cudaSuccess;
   Schedule &S = Y.base;
-  std::vector<int> dentry(v.n);
-  for (int i = 0; i < v.n; ++i) dentry[i] = S.src[S.dslot[i]];
+  split_schedule(S, v.n, v.nnz);
   std::vector<unsigned> word;
   std::vector<int> src;
-  int L = 0;
-  const int lanes = kind == kOne ? 32 : Lc;
-  if (kind != kPlain) {
-    if (kind == kOne) split_schedule(S, v.n, v.nnz);
-    L = sched::align(v.n, row_chains(S, v.rp), lanes, kind == kOne ? S.L2 : S.L, word, src);
-  }
-  if (L == 0 && kind == kOne) {
+  int L = sched::align(v.n, row_chains(S, v.rp), 32, S.L2, word, src);
+  if (L == 0) {
     L = S.L2;
     word = S.words2;
     src.assign(word.size(), -1);
     for (int k = 0; k < v.nnz; ++k) src[S.dst2[k]] = k;
-  } else if (L == 0) {
-    L = S.L;
-    word = S.words;
-    src = S.src;
   }
-  const cudaError_t e = upload_slots(to, lanes, L, v.nnz, word, src, dentry);
-  if (e != cudaSuccess) to = Slots();
+  Upload up;
+  Slots one;
+  add_slots(one, up, 32, L, v.nnz, word, src, Y.slots[kPlain].dentry);
+  const cudaError_t e = up.commit(&Y.block_one);
+  if (e == cudaSuccess) to = one;
   return e;
 }
 
 void free_view(View &v) {
-  for (auto &kv : v.sched)
-    for (Slots &S : kv.second.slots) S.release();
+  for (auto &kv : v.sched) {
+    cudaFree(kv.second.block);
+    cudaFree(kv.second.block_one);
+  }
   v.sched.clear();
 }
 
@@ -967,8 +971,8 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 // single_from, ngroups (tickets) and the split schedule's arguments; leaves
 // the launch without single tickets when the split schedule does not fit
 // the warp's region.
-cudaError_t set_single_tickets(camp_solver_t h, View &v, WarpArgs &a, int wpb, int occ,
-                               bool shared, cudaStream_t st) {
+cudaError_t set_single_tickets(camp_solver_t h, const View &v, Layout &Y, WarpArgs &a, int wpb,
+                               int occ, bool shared, cudaStream_t st) {
   const int pairs = a.ngroups;
   a.single_from = pairs;
   a.sched2 = nullptr;
@@ -983,7 +987,7 @@ cudaError_t set_single_tickets(camp_solver_t h, View &v, WarpArgs &a, int wpb, i
   }
   if (R == 0) return cudaSuccess;
   const Slots *S = nullptr;
-  const cudaError_t e = view_schedule(v, 16, kOne, st, nullptr, &S);
+  const cudaError_t e = one_slots(v, Y, st, &S);
   if (e != cudaSuccess) return e;
   const size_t need =
       ((size_t)(S->L * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
@@ -1031,9 +1035,9 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
       return fail(CAMP_EUNSUPPORTED, "n=%d needs %d rows per lane at %d lanes per cell (max %d)",
                   v.n, E, Lc, kMaxE);
     Layout *Y = nullptr;
-    const Slots *S = nullptr;
-    e = view_schedule(v, Lc, kAligned, st, &Y, &S);
+    e = view_schedule(v, Lc, &Y);
     if (e != cudaSuccess) return cuda_fail(e, "schedule upload");
+    const Slots *S = &Y->slots[kAligned];
     int wpb = h->wpb > 0 ? h->wpb : 4;
     int segA = 0, segV = 0, segStride = 0;
     size_t smem = warp_smem(v, Lc, S->L, wpb, &segA, &segV, &segStride);
@@ -1065,7 +1069,7 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
     e = warp_occupancy(E, Lc, kTicketsPack, wpb, smem, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy");
     if (occ < 1) occ = 1;
-    if ((e = set_single_tickets(h, v, a, wpb, occ, queue_slot != 0, st)) != cudaSuccess)
+    if ((e = set_single_tickets(h, v, *Y, a, wpb, occ, queue_slot != 0, st)) != cudaSuccess)
       return cuda_fail(e, "schedule upload");
     if (tickets_of(a) != kTicketsPack) {
       e = warp_occupancy(E, Lc, tickets_of(a), wpb, smem, &occ);
@@ -1668,7 +1672,8 @@ int4 with_double(double v, int z, int w) {
 }
 
 // The device tables (MechTables) of the handle's mechanism for Lc lanes per
-// cell on the slots S.
+// cell on the slots S, always the aligned ones of that lane count (the tables
+// hold their places).
 cudaError_t mech_terms(Mechanism &mech, int n, int Lc, const Slots &S, MechTerms **out) {
   auto it = mech.by_lanes.find(Lc);
   if (it != mech.by_lanes.end()) {
@@ -1804,9 +1809,8 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
   if (Lc == 0 || E > 8)
     return fail(CAMP_EUNSUPPORTED, "fused assembly supports at most 8 rows per lane (n=%d)", v.n);
   Layout *Y = nullptr;
-  const Slots *S = nullptr;
-  if ((e = view_schedule(v, Lc, kAligned, h->stream, &Y, &S)) != cudaSuccess)
-    return cuda_fail(e, "schedule upload");
+  if ((e = view_schedule(v, Lc, &Y)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+  const Slots *S = &Y->slots[kAligned];
   if (S->L > 2047) return fail(CAMP_EUNSUPPORTED, "more than 2047 slots per lane");
   MechTerms *T = nullptr;
   if ((e = mech_terms(h->mech, v.n, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
@@ -1945,9 +1949,9 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
   if (Lc == 0) return fail(CAMP_EUNSUPPORTED, "no warp arrangement fits n=%d", v.n);
   const int E = (v.n + Lc - 1) / Lc;
   if (E > kMaxE) return fail(CAMP_EUNSUPPORTED, "n=%d too large for %d lanes per cell", v.n, Lc);
-  const Slots *S = nullptr;
-  if ((e = view_schedule(v, Lc, kPlain, h->stream, nullptr, &S)) != cudaSuccess)
-    return cuda_fail(e, "schedule upload");
+  Layout *Y = nullptr;
+  if ((e = view_schedule(v, Lc, &Y)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+  const Slots *S = &Y->slots[kPlain];
   // FP64 A in shared memory unless that costs resident warps (then the
   // outer residual product reads it through L1)
   const int wpb0 = h->wpb > 0 ? h->wpb : 4;
@@ -2157,9 +2161,9 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
     View &v = h->fwd;
     int Lc = 1;
     while ((v.n + Lc - 1) / Lc > E) Lc *= 2;
-    const Slots *S = nullptr;
-    if ((e = view_schedule(v, Lc, kAligned, b->stream, nullptr, &S)) != cudaSuccess)
-      return cuda_fail(e, "schedule upload");
+    Layout *Y = nullptr;
+    if ((e = view_schedule(v, Lc, &Y)) != cudaSuccess) return cuda_fail(e, "schedule upload");
+    const Slots *S = &Y->slots[kAligned];
     WarpArgs &a = args.m[q];
     a.cells = cells[m]; a.n = v.n; a.nnz = v.nnz;
     a.Lc = Lc; a.log2Lc = ilog2(Lc); a.k = 32 / Lc;
