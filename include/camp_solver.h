@@ -100,8 +100,17 @@ camp_status camp_solver_create(camp_solver_t *out, int n, int nnz,
 /* Free the handle and its device memory (synchronises its stream first). */
 camp_status camp_solver_destroy(camp_solver_t h);
 
-/* Stream for subsequent calls: a cudaStream_t passed as void* (NULL = legacy
- * default stream). */
+/*
+ * Stream for subsequent calls: a cudaStream_t passed as void* (NULL = legacy
+ * default stream).
+ * Calls on a capturing stream: a handle allocates on the first use of a lane
+ * count in an orientation (and, with an ordering, on the first use of a batch
+ * size), of a mechanism's tables and of the host pipeline.  Capture modes that
+ * forbid allocation therefore need, before the capture, one call of the same
+ * entry point and orientation on a batch at least as large; calls of one entry
+ * point that differ in batch size only then need no other preparation, and a
+ * captured call launches the kernels that the same call launches outside one.
+ */
 camp_status camp_solver_set_stream(camp_solver_t h, void *stream);
 
 /*

@@ -338,20 +338,18 @@ struct Slots {
   int *d_dentry = nullptr;   // [n] A entry of each row's diagonal
 };
 
-// The layouts of one lane count.  The plain and the aligned one are built
-// together when the lane count is first used, so which of them a call runs
-// never depends on the calls before it, or on whether its stream captures a
-// graph (where nothing can be allocated); kOne when a small batch first needs
-// it (L 0: not yet).
+// The layouts of one lane count, built together when it is first used: which
+// of them a call runs never depends on the calls before it, or on whether its
+// stream captures a graph (where nothing can be allocated).
 enum Kind {
   kPlain = 0,    // the schedule as built (the refinement kernel)
   kAligned = 1,  // its rows aligned (align.h), where that takes no more slots
-  kOne = 2,      // at 16 lanes: the cell alone on 32 lanes
+  kOne = 2,      // at 16 lanes and up to kRegVecMaxE rows per lane: the cell
+                 // alone on 32 lanes (L 0 otherwise)
 };
 struct Layout {
-  Schedule base;
   Slots slots[3];
-  void *block = nullptr, *block_one = nullptr;  // the slots' device arrays
+  void *block = nullptr;  // the slots' device arrays
   // automatic warps per block, found once per kernel kind (0: not yet):
   // plain solve, fused assembly, Newton corrector
   int auto_wpb[3] = {0, 0, 0};
@@ -551,16 +549,27 @@ cudaError_t view_schedule(View &v, int Lc, Layout **out) {
   auto it = v.sched.find(Lc);
   if (it == v.sched.end()) {
     Layout Y;
-    Y.base = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
-    const Schedule &S = Y.base;
+    Schedule S = build_schedule(v.n, v.rp, v.ci, v.perm, v.diag, Lc);
+    const sched::RowChains ch = row_chains(S, v.rp);
     std::vector<int> dentry(v.n);
     for (int i = 0; i < v.n; ++i) dentry[i] = S.src[S.dslot[i]];
-    std::vector<unsigned> word;
-    std::vector<int> src;
-    const int L = sched::align(v.n, row_chains(S, v.rp), Lc, S.L, word, src);
     Upload up;
     add_slots(Y.slots[kPlain], up, Lc, S.L, v.nnz, S.words, S.src, dentry);
+    std::vector<unsigned> word;
+    std::vector<int> src;
+    const int L = sched::align(v.n, ch, Lc, S.L, word, src);
     if (L) add_slots(Y.slots[kAligned], up, Lc, L, v.nnz, word, src, dentry);
+    if (Lc == 16 && v.n <= 16 * kRegVecMaxE) {
+      split_schedule(S, v.n, v.nnz);
+      int L2 = sched::align(v.n, ch, 32, S.L2, word, src);
+      if (L2 == 0) {
+        L2 = S.L2;
+        word = S.words2;
+        src.assign(word.size(), -1);
+        for (int k = 0; k < v.nnz; ++k) src[S.dst2[k]] = k;
+      }
+      add_slots(Y.slots[kOne], up, 32, L2, v.nnz, word, src, dentry);
+    }
     const cudaError_t e = up.commit(&Y.block);
     if (e != cudaSuccess) return e;
     if (!L) Y.slots[kAligned] = Y.slots[kPlain];
@@ -570,39 +579,8 @@ cudaError_t view_schedule(View &v, int Lc, Layout **out) {
   return cudaSuccess;
 }
 
-// The layout of a cell alone on 32 lanes; left empty (L 0) while st captures
-// a graph.
-cudaError_t one_slots(const View &v, Layout &Y, cudaStream_t st, const Slots **slots) {
-  Slots &to = Y.slots[kOne];
-  *slots = &to;
-  if (to.L) return cudaSuccess;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap != cudaStreamCaptureStatusNone)
-    return cudaSuccess;
-  Schedule &S = Y.base;
-  split_schedule(S, v.n, v.nnz);
-  std::vector<unsigned> word;
-  std::vector<int> src;
-  int L = sched::align(v.n, row_chains(S, v.rp), 32, S.L2, word, src);
-  if (L == 0) {
-    L = S.L2;
-    word = S.words2;
-    src.assign(word.size(), -1);
-    for (int k = 0; k < v.nnz; ++k) src[S.dst2[k]] = k;
-  }
-  Upload up;
-  Slots one;
-  add_slots(one, up, 32, L, v.nnz, word, src, Y.slots[kPlain].dentry);
-  const cudaError_t e = up.commit(&Y.block_one);
-  if (e == cudaSuccess) to = one;
-  return e;
-}
-
 void free_view(View &v) {
-  for (auto &kv : v.sched) {
-    cudaFree(kv.second.block);
-    cudaFree(kv.second.block_one);
-  }
+  for (auto &kv : v.sched) cudaFree(kv.second.block);
   v.sched.clear();
 }
 
@@ -971,13 +949,13 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 // single_from, ngroups (tickets) and the split schedule's arguments; leaves
 // the launch without single tickets when the split schedule does not fit
 // the warp's region.
-cudaError_t set_single_tickets(camp_solver_t h, const View &v, Layout &Y, WarpArgs &a, int wpb,
-                               int occ, bool shared, cudaStream_t st) {
+void set_single_tickets(camp_solver_t h, const Slots &S, WarpArgs &a, int wpb, int occ,
+                        bool shared) {
   const int pairs = a.ngroups;
   a.single_from = pairs;
   a.sched2 = nullptr;
+  if (S.L == 0 || h->single_tail == 0) return;
   const int E16 = (a.n + 15) / 16;
-  if (a.Lc != 16 || a.k != 2 || E16 > kRegVecMaxE || h->single_tail == 0) return cudaSuccess;
   const long resident = (long)h->sms * occ * wpb;  // warps the GPU holds at once
   int R = 0;
   if (h->single_tail > 0) {
@@ -985,24 +963,20 @@ cudaError_t set_single_tickets(camp_solver_t h, const View &v, Layout &Y, WarpAr
   } else if (shared ? 3L * pairs <= resident : 4L * pairs <= 3L * resident) {
     R = pairs;  // a small batch: every cell alone, each warp nearly so
   }
-  if (R == 0) return cudaSuccess;
-  const Slots *S = nullptr;
-  const cudaError_t e = one_slots(v, Y, st, &S);
-  if (e != cudaSuccess) return e;
+  if (R == 0) return;
   const size_t need =
-      ((size_t)(S->L * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
-  if (S->L == 0 || need > 2 * (size_t)a.segStride) return cudaSuccess;
+      ((size_t)(S.L * 32 + 1) & ~(size_t)1) + 3 * (size_t)(((16 * E16 + 1) + 1) & ~1);
+  if (need > 2 * (size_t)a.segStride) return;
   const int P = pairs - R;
   a.single_from = P;
   a.ngroups = P + std::max(0, a.cells - 2 * P);
-  a.L2 = S->L;
-  a.sched2 = S->d_words;
-  a.dst2 = S->d_dst;
-  a.pads2 = S->d_pads;
-  a.npads2 = S->npads;
-  a.dslot2 = S->d_dslot;
-  memcpy(a.ends2, S->ends, sizeof a.ends2);
-  return cudaSuccess;
+  a.L2 = S.L;
+  a.sched2 = S.d_words;
+  a.dst2 = S.d_dst;
+  a.pads2 = S.d_pads;
+  a.npads2 = S.npads;
+  a.dslot2 = S.d_dslot;
+  memcpy(a.ends2, S.ends, sizeof a.ends2);
 }
 
 camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
@@ -1069,8 +1043,7 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
     e = warp_occupancy(E, Lc, kTicketsPack, wpb, smem, &occ);
     if (e != cudaSuccess) return cuda_fail(e, "occupancy");
     if (occ < 1) occ = 1;
-    if ((e = set_single_tickets(h, v, *Y, a, wpb, occ, queue_slot != 0, st)) != cudaSuccess)
-      return cuda_fail(e, "schedule upload");
+    set_single_tickets(h, Y->slots[kOne], a, wpb, occ, queue_slot != 0);
     if (tickets_of(a) != kTicketsPack) {
       e = warp_occupancy(E, Lc, tickets_of(a), wpb, smem, &occ);
       if (e != cudaSuccess) return cuda_fail(e, "occupancy");

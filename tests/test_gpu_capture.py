@@ -106,3 +106,22 @@ def test_captured_refinement_runs_the_refinement_layout(camp, cuda):
         nodes.append(_captured(lambda: s.solve_mixed(A, b)))
         s.close()
     assert nodes[0] and nodes[0] == nodes[1]
+
+
+@pytest.mark.parametrize("transpose", [False, True])
+def test_captured_small_batch_runs_single_cells(camp, cuda, transpose):
+    """A small batch at 16 lanes per cell, captured after one large solve, launches
+    what it launches eagerly: every cell alone on a warp."""
+    import torch
+    m = synth.make_mechanism(80, 200, 602)
+    cb = synth.make_cells(m, 5000, 603, gamma=(1e-4, 1e-1))
+    A, b = (torch.as_tensor(v, device=cuda) for v in (cb.A_vals, cb.b))
+    nodes = []
+    for first in (5000, 64):
+        s = camp.Solver(m.row_ptr, m.col_idx)
+        s.solve(A[:first], b[:first], transpose=transpose)
+        nodes.append(_captured(lambda: s.solve(A[:64], b[:64], transpose=transpose)))
+        s.set_single_tail(0)
+        pairs = _captured(lambda: s.solve(A[:64], b[:64], transpose=transpose))
+        s.close()
+    assert nodes[0] and nodes[0] == nodes[1] and nodes[0] != pairs
