@@ -161,10 +161,11 @@ camp_status camp_solver_set_arrangement(camp_solver_t h, int arrangement,
  *      the host from the counts of that full read (copied back without
  *      blocking).  Device scratch: 8 bytes per cell plus 4 per row.
  *      Solves on other streams (camp_solver_solve_host's chunks) and launches
- *      with at most one group per SM sub-partition, which end with their hardest
- *      cell in any order, use index order; launches whose warp regions cannot lend the ordering 2,576
- *      bytes of shared memory, or whose cooperative launch the GPU refuses
- *      (fewer SMs available than its occupancy query counts), use mode 2.  Under stream capture the
+ *      whose groups all start at once, at most one per SM sub-partition (they
+ *      end with their hardest cell in any order), use index order; launches
+ *      whose warp regions cannot lend the ordering 2,576 bytes of shared
+ *      memory, or whose cooperative launch the GPU refuses (fewer SMs available
+ *      than its occupancy query counts), use mode 2.  Under stream capture the
  *      last picked rows are used as they are (allocate first: run one solve
  *      before capturing).  Every wait of the launch is bounded (about a
  *      second).  If one runs out, the same launch marks every cell of the
@@ -297,8 +298,8 @@ camp_status camp_batch_set_config(camp_batch_t b, int rows_per_lane,
  * same difficulty estimate and classes as camp_solver_set_ordering (a
  * classify and a scatter launch over all mechanisms, part of the batch's
  * graph; device scratch of 9 bytes per cell plus 256 bytes per mechanism);
- * 0 keeps index order, as does a batch with at most one work item per SM
- * sub-partition.  Results are bitwise the same either way.
+ * 0 keeps index order, as does a batch whose work items all start at once, at
+ * most one per SM sub-partition.  Results are bitwise the same either way.
  * CAMP_EINVAL for other values.
  */
 camp_status camp_batch_set_ordering(camp_batch_t b, int ordering);

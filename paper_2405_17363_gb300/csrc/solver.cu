@@ -811,21 +811,28 @@ camp_status ensure_order_capacity(camp_solver_t h, int cells, cudaStream_t st) {
   return CAMP_OK;
 }
 
-// Whether ordering the cells can shorten a launch: with at most one group per
-// SM sub-partition every group starts at once on an FP64 unit of its own, and
-// the launch ends with its hardest cell whatever the order, so the prologue
-// (and the cooperative launch) would only delay it (64 cells of 30 species:
-// 35.6 us with it, 32.5 without; 600 cells of 80 species: 45.5 and 42.0).
-bool worth_ordering(camp_solver_t h, int ngroups) { return ngroups > 4 * h->sms; }
+// Whether ordering the cells can shorten a launch of `groups` groups with
+// `warps` resident warps per SM: not when every group starts at once on an FP64
+// unit of its own (at most one per SM sub-partition), for the launch then ends
+// with its hardest cell whatever the order, and the prologue (and the
+// cooperative launch) would only delay it (64 cells of 30 species: 35.6 us with
+// it, 32.5 without; 600 cells of 80 species: 45.5 and 42.0).  Cells so large
+// that an SM holds fewer than four warps start in several waves: there the
+// hardest ones have to come first (107 species, 7,653 entries, two warps per SM, 608
+// cells: 1,288 us in index order, 867 in order).
+bool worth_ordering(int sms, int warps, int groups) {
+  return groups > sms * std::min(4, warps);
+}
 
 // In-launch ordering of the fused-assembly and Newton launches (orderings 1
 // and 2): cells classified by gamma, as the plain launch classifies them by
 // its sampled diagonal (there is no matrix before a cell is assembled).
 // Leaves a unordered when the warp regions cannot lend the ordering its
 // shared memory.
-camp_status setup_gamma_ordering(camp_solver_t h, WarpArgs &a, size_t smem_free,
+camp_status setup_gamma_ordering(camp_solver_t h, WarpArgs &a, int warps, size_t smem_free,
                                  cudaStream_t st) {
-  if (!h->ordering || !worth_ordering(h, a.ngroups) || smem_free < kOrdSmemBytes) return CAMP_OK;
+  if (!h->ordering || !worth_ordering(h->sms, warps, a.ngroups) || smem_free < kOrdSmemBytes)
+    return CAMP_OK;
   camp_status rs = ensure_order_capacity(h, a.cells, st);
   if (rs != CAMP_OK) return rs;
   cudaError_t e;
@@ -858,14 +865,15 @@ void drop_gamma_ordering(WarpArgs &a) {
 // launch, borrowing kOrdSmemBytes of the warp regions (smem_free bytes of
 // them) before they are used; ordering 2, or 1 where that does not fit, runs
 // the separate classify and scatter pass.  Fills the order fields of a
-// (WarpArgs or MixedArgs; a.cells, a.ngroups set); *calibrate tells the
-// caller to read the peak-row counts back after the launch.
+// (WarpArgs or MixedArgs; a.cells, a.ngroups set) of a launch with `warps`
+// resident warps per SM; *calibrate tells the caller to read the peak-row
+// counts back after the launch.
 template <class Args>
-camp_status setup_ordering(camp_solver_t h, Args &a, const double *A_vals, size_t smem_free,
-                           cudaStream_t st, bool *calibrate) {
+camp_status setup_ordering(camp_solver_t h, Args &a, const double *A_vals, int warps,
+                           size_t smem_free, cudaStream_t st, bool *calibrate) {
   const int cells = a.cells;
   *calibrate = false;
-  if (!h->ordering || !worth_ordering(h, a.ngroups)) return CAMP_OK;
+  if (!h->ordering || !worth_ordering(h->sms, warps, a.ngroups)) return CAMP_OK;
   cudaError_t e = cudaSuccess;
   const bool inl = h->ordering == 1 && smem_free >= kOrdSmemBytes;
   if (inl) {
@@ -1050,8 +1058,8 @@ camp_status do_solve(camp_solver_t h, int cells, const double *A_vals,
       if (occ < 1) occ = 1;
     }
     if (queue_slot == 0) {
-      const camp_status rs = setup_ordering(h, a, A_vals, smem - sched_smem_bytes(S->L * Lc), st,
-                                            &calibrate);
+      const camp_status rs = setup_ordering(h, a, A_vals, occ * wpb,
+                                            smem - sched_smem_bytes(S->L * Lc), st, &calibrate);
       if (rs != CAMP_OK) return rs;
     }
     const int need = (a.ngroups + wpb - 1) / wpb;
@@ -1841,7 +1849,7 @@ camp_status camp_solver_assemble_solve(camp_solver_t h, int cells,
   if ((e = assemble_occupancy(E, a.Lc, kTicketsPack, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min((a.ngroups + wpb - 1) / wpb, h->sms * occ));
-  rc = setup_gamma_ordering(h, a, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
+  rc = setup_gamma_ordering(h, a, occ * wpb, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
   if (rc != CAMP_OK) return rc;
   set_wave(a, grid, wpb);
   e = launch_cooperative(h, a.ord_ws != nullptr,
@@ -1888,7 +1896,7 @@ camp_status camp_solver_newton_solve(camp_solver_t h, int cells,
   if ((e = newton_occupancy(E, a.Lc, kTicketsPack, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min((a.ngroups + wpb - 1) / wpb, h->sms * occ));
-  rc = setup_gamma_ordering(h, a, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
+  rc = setup_gamma_ordering(h, a, occ * wpb, smem - sched_smem_bytes(a.L * a.Lc), h->stream);
   if (rc != CAMP_OK) return rc;
   set_wave(a, grid, wpb);
   e = launch_cooperative(h, a.ord_ws != nullptr,
@@ -1962,14 +1970,14 @@ camp_status camp_solver_solve_mixed(camp_solver_t h, int cells,
   // choice above 48 species) its prologue costs more than hardest-first saves
   // (131 against 125 us at 80 species x 10,000 cells).
   bool calibrate = false;
-  if (a.k > 1) {
-    const camp_status rs = setup_ordering(h, a, A_vals, smem - sched_smem_bytes(S->L * Lc),
-                                          h->stream, &calibrate);
-    if (rs != CAMP_OK) return rs;
-  }
   int occ = 0;
   if ((e = mixed_occupancy(E, Lc, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "occupancy");
   if (occ < 1) occ = 1;
+  if (a.k > 1) {
+    const camp_status rs = setup_ordering(h, a, A_vals, occ * wpb,
+                                          smem - sched_smem_bytes(S->L * Lc), h->stream, &calibrate);
+    if (rs != CAMP_OK) return rs;
+  }
   const int need = (a.ngroups + wpb - 1) / wpb;
   const int grid = std::max(1, std::min(need, h->sms * occ));
   set_wave(a, grid, wpb);
@@ -2157,43 +2165,6 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
   args.total_items = items;
   args.warp_doubles = warp_doubles;
   if (items == 0) return CAMP_OK;
-  // hardest first within each mechanism (mechanisms stay largest first)
-  BatchOrderArgs oa;
-  memset(&oa, 0, sizeof oa);
-  oa.nmech = b->nmech;
-  for (int q = 0; q < b->nmech; ++q) {
-    const int m = order[q];
-    oa.A[q] = A_vals[m];
-    oa.diag[q] = b->mech[m]->fwd.d_diag;
-    oa.n[q] = b->mech[m]->n;
-    oa.nnz[q] = b->mech[m]->nnz;
-    oa.cell_begin[q + 1] = oa.cell_begin[q] + cells[m];
-  }
-  const int total_cells = oa.cell_begin[b->nmech];
-  // (see worth_ordering: with every item running at once the order is no use,
-  // and its three nodes come before the solve)
-  const bool ordered = b->ordering && items > 4 * b->sms;
-  const size_t cnt_bytes = (size_t)b->nmech * kOrdClasses * sizeof(int);
-  if (ordered) {
-    if ((size_t)total_cells > b->ord_cap) {
-      cudaFree(b->d_ord);
-      b->d_ord = nullptr;
-      b->ord_cap = 0;
-      // counters, the order and the places (4 bytes per cell each), then the
-      // classes (1 byte per cell)
-      if ((e = cudaMalloc(&b->d_ord, cnt_bytes + (size_t)total_cells * 9)) != cudaSuccess)
-        return fail(CAMP_ENOMEM, "batch ordering scratch: %s", cudaGetErrorString(e));
-      b->ord_cap = (size_t)total_cells;
-    }
-    oa.counts = (int *)b->d_ord;
-    oa.order = (int *)(b->d_ord + cnt_bytes);
-    oa.pos = oa.order + b->ord_cap;
-    oa.cls = b->d_ord + cnt_bytes + b->ord_cap * 8;
-    for (int q = 0; q < b->nmech; ++q) args.m[q].order = oa.order + oa.cell_begin[q];
-  }
-  const int ogrid = std::max(1, (total_cells + kBatchOrderPiece - 1) / kBatchOrderPiece);
-  const int sgrid = (total_cells + 255) / 256;
-  void *oparams[] = {&oa};
   int wpb = b->wpb > 0 ? b->wpb : 4;
   size_t smem = (size_t)wpb * warp_doubles * 8;
   while (smem > b->smem_optin && wpb > 1) smem = (size_t)(--wpb) * warp_doubles * 8;
@@ -2216,6 +2187,41 @@ camp_status camp_batch_solve(camp_batch_t b, const int *cells,
   if ((e = batch_prepare(E, asmem, wpb, smem, &occ)) != cudaSuccess) return cuda_fail(e, "batch occupancy");
   if (occ < 1) occ = 1;
   const int grid = std::max(1, std::min(b->sms * occ, (items + wpb - 1) / wpb));
+  // hardest first within each mechanism (mechanisms stay largest first)
+  BatchOrderArgs oa;
+  memset(&oa, 0, sizeof oa);
+  oa.nmech = b->nmech;
+  for (int q = 0; q < b->nmech; ++q) {
+    const int m = order[q];
+    oa.A[q] = A_vals[m];
+    oa.diag[q] = b->mech[m]->fwd.d_diag;
+    oa.n[q] = b->mech[m]->n;
+    oa.nnz[q] = b->mech[m]->nnz;
+    oa.cell_begin[q + 1] = oa.cell_begin[q] + cells[m];
+  }
+  const int total_cells = oa.cell_begin[b->nmech];
+  const bool ordered = b->ordering && worth_ordering(b->sms, occ * wpb, items);
+  const size_t cnt_bytes = (size_t)b->nmech * kOrdClasses * sizeof(int);
+  if (ordered) {
+    if ((size_t)total_cells > b->ord_cap) {
+      cudaFree(b->d_ord);
+      b->d_ord = nullptr;
+      b->ord_cap = 0;
+      // counters, the order and the places (4 bytes per cell each), then the
+      // classes (1 byte per cell)
+      if ((e = cudaMalloc(&b->d_ord, cnt_bytes + (size_t)total_cells * 9)) != cudaSuccess)
+        return fail(CAMP_ENOMEM, "batch ordering scratch: %s", cudaGetErrorString(e));
+      b->ord_cap = (size_t)total_cells;
+    }
+    oa.counts = (int *)b->d_ord;
+    oa.order = (int *)(b->d_ord + cnt_bytes);
+    oa.pos = oa.order + b->ord_cap;
+    oa.cls = b->d_ord + cnt_bytes + b->ord_cap * 8;
+    for (int q = 0; q < b->nmech; ++q) args.m[q].order = oa.order + oa.cell_begin[q];
+  }
+  const int ogrid = std::max(1, (total_cells + kBatchOrderPiece - 1) / kBatchOrderPiece);
+  const int sgrid = (total_cells + 255) / 256;
+  void *oparams[] = {&oa};
   void *kparams[] = {&args};
   cudaKernelNodeParams kp;
   memset(&kp, 0, sizeof kp);
