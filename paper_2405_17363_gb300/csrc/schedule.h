@@ -87,17 +87,15 @@ inline int slot_cost(long j, int Lc, const unsigned *word, const int *entry) {
     const int M = pass ? 32 : G;          // residues
     const int span = pass ? 32 : G;       // lanes counted together
     for (int g0 = 0; g0 < Lc; g0 += span) {
-      int cols[32], ncol = 0, cnt[32];
+      int cols[32][32], cnt[32];  // distinct columns by residue
       for (int r = 0; r < M; ++r) cnt[r] = 0;
       for (int x = 0; x < span; ++x) {
         const size_t t = (size_t)j * Lc + g0 + x;
         if (entry[t] < 0) continue;
-        const int c = (int)(word[t] & 0x7ffu);
+        const int c = (int)(word[t] & 0x7ffu), r = c & (M - 1);
         bool dup = false;
-        for (int y = 0; y < ncol && !dup; ++y) dup = cols[y] == c;
-        if (dup) continue;
-        cols[ncol++] = c;
-        ++cnt[c % M];
+        for (int y = 0; y < cnt[r] && !dup; ++y) dup = cols[r][y] == c;
+        if (!dup) cols[r][cnt[r]++] = c;
       }
       int worst = 0;
       for (int r = 0; r < M; ++r) worst = cnt[r] > worst ? cnt[r] : worst;

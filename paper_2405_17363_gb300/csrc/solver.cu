@@ -818,8 +818,8 @@ camp_status ensure_order_capacity(camp_solver_t h, int cells, cudaStream_t st) {
 // cooperative launch) would only delay it (64 cells of 30 species: 35.6 us with
 // it, 32.5 without; 600 cells of 80 species: 45.5 and 42.0).  Cells so large
 // that an SM holds fewer than four warps start in several waves: there the
-// hardest ones have to come first (107 species, 7,653 entries, two warps per SM, 608
-// cells: 1,288 us in index order, 867 in order).
+// hardest ones have to come first (107 species, 7,653 entries, two warps per SM,
+// 608 cells: 1,288 us in index order, 867 in order).
 bool worth_ordering(int sms, int warps, int groups) {
   return groups > sms * std::min(4, warps);
 }
