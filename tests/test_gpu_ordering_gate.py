@@ -55,3 +55,41 @@ def test_cells_too_large_for_four_warps_are_ordered(camp, cuda):
     batch.close()
     other.close()
     s.close()
+
+
+# (species, reactions, call, cells per warp): all rows sampled (up to 8 species),
+# a sample of them, the refinement (several cells per warp), by gamma; single
+# cells (16 lanes, small batch) are a warp each
+@pytest.mark.parametrize("n,R,call,k", [(6, 12, "solve", 16), (30, 60, "solve", 4), (80, 200, "solve", 1),
+                                        (24, 60, "solve_mixed", 4), (80, 200, "assemble_solve", 2)])
+def test_small_ordered_launches_between_large_ones(camp, cuda, n, R, call, k):
+    """One group more than starts at once is ordered and one group fewer is not;
+    in a sequence of such launches and larger ones every mode gives bitwise the
+    results of index order (nothing left over from a launch misplaces a cell)."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    edge = 4 * sms * k
+    sizes = (edge + 1, 5 * edge + 7, edge, edge + 1, 2 * edge + 3, edge + k)
+    m = synth.make_mechanism(n, R, 710 + n)
+    cb = synth.make_cells(m, max(sizes), 711 + n, gamma=(1e-4, 1e-1))
+    A, b, conc, gam = (torch.as_tensor(v, device=cuda) for v in (cb.A_vals, cb.b, cb.conc, cb.gamma))
+    s = camp.Solver(m.row_ptr, m.col_idx)
+    s.set_mechanism(m.reactants[:, 0], m.reactants[:, 1], m.products, m.k)
+
+    def run(c):
+        if call == "assemble_solve":
+            return s.assemble_solve(conc[:c], gam[:c], b[:c])
+        return getattr(s, call)(A[:c], b[:c])
+
+    s.set_ordering(0)
+    want = [t.clone() for t in run(max(sizes))]
+    for mode in (1, 2, 1):
+        s.set_ordering(mode)
+        for c in sizes:
+            assert _same(run(c), [t[:c] for t in want]), (mode, c)
+    assert not s.get_fault()
+    if call != "assemble_solve":   # mode 2 of the others shows as launches of its own
+        s.set_ordering(2)
+        assert len(_captured(lambda: run(edge))) == 1
+        assert any("classify" in q[0] for q in _captured(lambda: run(edge + 1)))
+    s.close()
