@@ -132,11 +132,11 @@ camp_status camp_solver_set_stream(camp_solver_t h, void *stream);
  *   CAMP_ARR_AUTO : library choice.
  * With 16 lanes per cell (the automatic choice for 41 to 80 species), a
  * launch whose pairs would keep at most three quarters of the GPU's resident
- * warps busy (half at 49 to 56 species; a third up to 48 and in
- * camp_solver_solve_host's chunks) solves each cell alone on a warp instead, on
- * a split of the 16-lane layout that performs the same operations in the same
- * order: the results are bit for bit those of the pair solve, and a batch of
- * up to some 600 cells of 80 species finishes about a quarter sooner.
+ * warps busy (a third up to 48 species and in camp_solver_solve_host's chunks)
+ * solves each cell alone on a warp instead, on a split of the 16-lane layout
+ * that performs the same operations in the same order: the results are bit for
+ * bit those of the pair solve, and a batch of up to some 600 cells of 80
+ * species finishes about a quarter sooner.
  * Unused arguments are ignored.  Returns CAMP_EINVAL for unsupported values.
  */
 camp_status camp_solver_set_arrangement(camp_solver_t h, int arrangement,

@@ -950,18 +950,18 @@ cudaError_t launch_cooperative(camp_solver_t h, bool cooperative, Launch launch)
 // every pair when the pairs would keep at most a share of the resident warps
 // busy (a lone warp's latency decides such a launch), else none (at full load
 // one cell per warp costs about 13 % more per cell).  The fewer rows a lane
-// has, the less of an iteration is its rows' work and the more a pair shares,
-// so the share falls with them: three quarters above 56 rows, half above 48,
-// else a third.  us, alone against pairs, 152 SMs x 12 warps: 80 species x 600
-// easy cells 37 and 50, x 2,700 74 and 76 (stiff 747 and 902), but x 4,000 103
-// and 87; 49 species x 1,824 43 and 44 (stiff 524 and 674), x 2,432 54 and 45
-// (stiff 569 and 614); 41 species x 608 29 and 31 (stiff 779 and 848), x 1,216
-// 40 and 33 (stiff 806 and 848), x 2,200 54 and 42 (stiff 2,267 and 2,382).  A
-// third too when the launch shares the GPU with others (`shared`: the chunks of
-// the host-memory pipeline).  camp_solver_set_single_tail overrides it.  Sets
-// single_from, ngroups (tickets) and the split layout's arguments; leaves the
-// launch without single tickets when that layout does not fit the warp's
-// region.
+// has, the less of an iteration is its rows' work and the more a pair shares:
+// three quarters with four or five rows per lane, a third with fewer (up to 48
+// rows).  us, alone against pairs, 152 SMs x 12 warps: 80 species x 600 easy
+// cells 37 and 50, x 2,700 74 and 76 (stiff 747 and 902), but x 4,000 103 and
+// 87; 49 to 54 species, two mechanisms each, x 1,900 to 2,736: alone 10 %
+// faster on average (stiff 15 %), 18 % slower at worst; 41 species x 608 29 and
+// 31 (stiff 779 and 848), x 1,216 40 and 33 (stiff 806 and 848), x 2,200 54 and
+// 42 (stiff 2,267 and 2,382).  A third too when the launch shares the GPU with
+// others (`shared`: the chunks of the host-memory pipeline).
+// camp_solver_set_single_tail overrides it.  Sets single_from, ngroups
+// (tickets) and the split layout's arguments; leaves the launch without single
+// tickets when that layout does not fit the warp's region.
 void set_single_tickets(camp_solver_t h, const Slots &S, WarpArgs &a, int wpb, int occ,
                         bool shared) {
   const int pairs = a.ngroups;
@@ -970,7 +970,7 @@ void set_single_tickets(camp_solver_t h, const Slots &S, WarpArgs &a, int wpb, i
   if (S.L == 0 || h->single_tail == 0) return;
   const int E16 = (a.n + 15) / 16;
   const long resident = (long)h->sms * occ * wpb;  // warps the GPU holds at once
-  const long twelfths = shared || a.n <= 48 ? 4 : a.n <= 56 ? 6 : 9;
+  const long twelfths = shared || E16 <= 3 ? 4 : 9;
   int R = 0;
   if (h->single_tail > 0) {
     R = std::min(pairs, h->single_tail);

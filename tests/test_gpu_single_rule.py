@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 # rows, twelfths of the resident warps
-@pytest.mark.parametrize("n,share", [(41, 4), (48, 4), (49, 6), (56, 6), (57, 9), (80, 9)])
+@pytest.mark.parametrize("n,share", [(41, 4), (48, 4), (49, 9), (80, 9)])
 def test_share_of_the_warps_that_pairs_may_fill(cuda, n, share):
     import torch
     from paper_2405_17363_gb300 import camp
