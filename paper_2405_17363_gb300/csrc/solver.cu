@@ -210,7 +210,7 @@ struct Schedule {
   // 0: none); see split_schedule
   int L2 = 0;
   std::vector<unsigned> words2;  // [L2][32]
-  std::vector<int> dst2, padfrom2, dslot2;
+  std::vector<int> dst2;         // [nnz] split slot of each A entry
 };
 
 // The split schedule of a 16-lane schedule: one cell on all 32 lanes, lane v
@@ -219,9 +219,9 @@ struct Schedule {
 // exhaustively for up to 16 rows, else greedily longest first); every row
 // keeps its slots' order, so each row's sum is the same chain of
 // multiply-adds as in the pair solve; padding slots multiply zero by column
-// 0.  Fills L2, words2, dst2, padfrom2 and dslot2 (L2 stays 0 unless the
-// schedule is 16 lanes wide).
-void split_schedule(Schedule &S, int n, int nnz) {
+// 0.  Fills L2, words2 and dst2 (L2 stays 0 unless the schedule is 16 lanes
+// wide).
+void split_schedule(Schedule &S, int nnz) {
   if (S.Lc != 16 || S.L == 0) return;
   std::vector<std::vector<int>> rstart(16), rlen(16);
   std::vector<std::vector<char>> side(16);  // side[v][r]: row r of lane v goes to lane v + 16
@@ -270,10 +270,7 @@ void split_schedule(Schedule &S, int n, int nnz) {
   }
   S.L2 = L2;
   S.words2.assign((size_t)L2 * 32, 0u);
-  S.padfrom2.assign(32, 0);
   S.dst2.assign(nnz, -1);
-  S.dslot2.assign(n, -1);
-  std::vector<int> map16((size_t)S.L * 16, -1);
   for (int v = 0; v < 16; ++v) {
     int fill[2] = {0, 0};
     for (size_t r = 0; r < rlen[v].size(); ++r) {
@@ -283,15 +280,10 @@ void split_schedule(Schedule &S, int n, int nnz) {
         const size_t t16 = (size_t)(rstart[v][r] + q) * 16 + v;
         const size_t t2 = (size_t)fill[h]++ * 32 + lane;
         S.words2[t2] = S.words[t16];
-        map16[t16] = (int)t2;
         if (S.src[t16] >= 0) S.dst2[S.src[t16]] = (int)t2;
       }
     }
-    S.padfrom2[v] = fill[0];
-    S.padfrom2[v + 16] = fill[1];
   }
-  for (int r = 0; r < n; ++r)
-    if (S.dslot[r] >= 0) S.dslot2[r] = map16[S.dslot[r]];
 }
 
 Schedule build_schedule(int n, const std::vector<int> &rp,
@@ -560,7 +552,7 @@ cudaError_t view_schedule(View &v, int Lc, Layout **out) {
     const int L = sched::align(v.n, ch, Lc, S.L, word, src);
     if (L) add_slots(Y.slots[kAligned], up, Lc, L, v.nnz, word, src, dentry);
     if (Lc == 16 && v.n <= 16 * kRegVecMaxE) {
-      split_schedule(S, v.n, v.nnz);
+      split_schedule(S, v.nnz);
       int L2 = sched::align(v.n, ch, 32, S.L2, word, src);
       if (L2 == 0) {
         L2 = S.L2;
@@ -1169,7 +1161,7 @@ camp_status camp_schedule_build_split(int n, int nnz, const int *row_ptr,
     if (diag[i] < 0) return fail(CAMP_EPATTERN, "diagonal entry missing in row %d", i);
   }
   Schedule S = build_schedule(n, rp, ci, std::vector<int>(), diag, 16);
-  split_schedule(S, n, nnz);
+  split_schedule(S, nnz);
   *slots_per_lane = S.L2;
   if (words) {
     if ((long)S.L2 * 32 > (long)capacity_slots)
@@ -1198,7 +1190,7 @@ camp_status camp_schedule_build_aligned(int n, int nnz, const int *row_ptr, cons
     for (int k = rp[i]; k < rp[i + 1]; ++k)
       if (ci[k] == i) diag[i] = k;
   Schedule S = build_schedule(n, rp, ci, std::vector<int>(), diag, lanes_per_cell);
-  if (split) split_schedule(S, n, nnz);
+  if (split) split_schedule(S, nnz);
   const int lanes = split ? 32 : lanes_per_cell;
   std::vector<unsigned> word;
   std::vector<int> src;
@@ -1798,12 +1790,14 @@ static camp_status fused_args(camp_solver_t h, int cells, int extra_vectors, Occ
   Layout *Y = nullptr;
   if ((e = view_schedule(v, Lc, &Y)) != cudaSuccess) return cuda_fail(e, "schedule upload");
   const Slots *S = &Y->slots[kAligned];
-  if (S->L > 2047) return fail(CAMP_EUNSUPPORTED, "more than 2047 slots per lane");
-  MechTerms *T = nullptr;
-  if ((e = mech_terms(h->mech, v.n, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
   int wpb = h->wpb > 0 ? h->wpb : 4;
   int segA = 0, segV = 0, segStride = 0;
   size_t smem = warp_smem(v, Lc, S->L, wpb, &segA, &segV, &segStride, extra_vectors);
+  // the rate tables hold places of concentrations in 16 bits
+  if (segA + 2 * segV + v.n > 65536)
+    return fail(CAMP_EUNSUPPORTED, "%d slots per lane are too many for the mechanism tables", S->L);
+  MechTerms *T = nullptr;
+  if ((e = mech_terms(h->mech, v.n, Lc, *S, &T)) != cudaSuccess) return cuda_fail(e, "mechanism upload");
   while (smem > h->smem_optin && wpb > 1)
     smem = warp_smem(v, Lc, S->L, --wpb, &segA, &segV, &segStride, extra_vectors);
   if (smem > h->smem_optin) return fail(CAMP_EUNSUPPORTED, "cell does not fit in shared memory");
