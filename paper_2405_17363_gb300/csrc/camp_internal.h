@@ -8,7 +8,7 @@
 namespace camp {
 
 // SpMV schedule word of one slot (see build_schedule in solver.cu): 4 * col
-// (bits 16-31) | 4 * row (bits 2-11) | end (bit 0): the slot multiplies the
+// (bits 16-31) | 4 * row (bits 2-15) | end (bit 0): the slot multiplies the
 // gathered vector's entry col; on the last slot of a row (end) the running
 // sum is stored to row.  Four slots of a lane are one 16-byte load: slot j of
 // lane sl lies at word_pos(j, sl).  Alongside, src (same places) is the entry

@@ -299,10 +299,10 @@ __device__ __forceinline__ void mixed_body(const MixedArgs &a) {
 
 // FP32 and FP64 issue and shared memory are each about half busy, so resident
 // warps hide the rest: 20 per SM (96 registers), and 24 (80 registers) with up
-// to 3 rows per lane on 32 lanes, where nothing spills and A in FP64 is not
-// read through L1; 16 (128 registers) beyond 5 rows per lane.  16 / 20 / 24 warps: 150 species x 100,000 cells 1,919 /
-// 1,858 / 2,273 us, 80 x 10,000 117 / 112 / 105, 40 x 20,000 (16 lanes) 114 /
-// 113 / 123.
+// to 3 rows per lane on 32 lanes, where 4 bytes spill and A in FP64 is not read
+// through L1; 16 (128 registers) beyond 5 rows per lane.  16 / 20 / 24 warps:
+// 150 species x 100,000 cells 1,919 / 1,858 / 2,273 us, 80 x 10,000 117 / 112 /
+// 105, 40 x 20,000 (16 lanes) 114 / 113 / 123.
 template <int E, int LC>
 constexpr bool kMixedMany = E <= 3 && LC == 32;
 template <int E, int LC>

@@ -132,6 +132,13 @@ __device__ __forceinline__ void slot_end(unsigned w, T &acc, unsigned os) {
 // 65 per slot and warp with three or four warps per sub-partition either way.
 // (Two word sets and an unrolled pair of blocks: 81 alone, but the kernels
 // around it spilled: 183 us against 180 at 80 species x 10,000 cells.)
+// A pattern without an aligned layout (align.h finds none: dense ones, above
+// some 250 rows; and camp_solve_noalloc) runs it on the schedule as built, with
+// the mask set wherever rows end: in nearly every slot of a sparse pattern,
+// where spmv_flat below would be a little faster, in a few of a dense one, where
+// it would be slower (us a solve, this and spmv_flat: 400 species, 2,880
+// entries, 5,000 cells 666 and 646; 512, 3,997, 4,000 cells 900 and 870; 107,
+// 7,653, 2,000 cells 2,074 and 2,301; 40, 1,235, 5,000 cells 397 and 424).
 template <class T, class Lo, class Hi, class Last>
 __device__ __forceinline__ void spmv_slots(const SchedWord *__restrict__ sch,
                                            const unsigned *__restrict__ ends, int L, int Lc, int sl,

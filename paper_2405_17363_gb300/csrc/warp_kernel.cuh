@@ -599,7 +599,8 @@ __device__ __forceinline__ void solve_group(const WarpArgs &a, int g,
 // LC: lanes per cell at compile time (0: a.Lc).  TK: which tickets the launch
 // has (the plain solve at 16 lanes only; see WarpArgs::single_from).  Each
 // combination is a kernel of its own: one kernel holding all of them spilled
-// 520 bytes a thread at 5 rows per lane, where each alone spills 8 at most.
+// 520 bytes a thread at 5 rows per lane, where those of the automatic launches
+// spill nothing (the one with both kinds of tickets 20 bytes; Newton 44).
 template <int E, int SRC, int LC, int TK>
 __device__ __forceinline__ void plain_launch_body(const WarpArgs &a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
